@@ -222,11 +222,12 @@ typedef struct {
  * energy recorded; the step still completes.  The first step with species
  * larger than any stepped before grows the context's look-back scratch (one
  * allocation, synchronous); otherwise no allocation, no host synchronisation,
- * no host reads: the call can then be captured in a CUDA graph.  Each step
- * is one launch of the step kernel over every resident block of the GPU; on
- * the mixed path it is a cooperative launch, which starts only once all its
- * blocks fit on the GPU (kernels of other streams that hold SMs finish
- * first).
+ * no host reads: the call can then be captured in a CUDA graph.  Up to eight
+ * steps (one while launches are timed, see qp_profile_enable) are one launch
+ * of the step kernel over every resident block of the GPU; on the mixed path,
+ * and for more than one step, it is a cooperative launch, which starts only
+ * once all its blocks fit on the GPU (kernels of other streams that hold SMs
+ * finish first).
  * Returns QP_ERR_INVALID_ARG (nothing enqueued) for bad parameters, a
  * missing photon species while species emit, or a YEE2D grid with a NULL
  * component; QP_ERR_CUDA if a launch fails.  Overflow, table clamping and
@@ -599,7 +600,7 @@ int qp_reset_counters(qp_ctx *ctx, int32_t handle);
 
 /*
  * Kernel timing for benchmarks.  While enabled, qp_step and qp_batch_step
- * bracket each launch of the fused step kernel (one launch per step) with CUDA
+ * bracket each launch of the fused step kernel (one step a launch then) with CUDA
  * events recorded on the step's stream (events are owned by the context;
  * enabling clears earlier records).  qp_profile_read synchronises on the
  * recorded events and returns in ms[0] the summed device time in ms and in

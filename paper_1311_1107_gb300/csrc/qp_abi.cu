@@ -58,7 +58,7 @@ struct qp_ctx {
     size_t chain_words = 0;           // words per chain
     double *d_diag = nullptr;         // partials + final
     double *d_stash = nullptr;        // append records of qp_step launches
-    size_t stash_blocks = 0;          // blocks the stash is sized for
+    size_t stash_bytes = 0;
     void *d_fuse = nullptr;           // scratch of qp_step_fused
     size_t fuse_bytes = 0;
     void *d_coal = nullptr;           // scratch of qp_coalesce_photons
@@ -180,13 +180,6 @@ int ensure_chain(qp_ctx *c, size_t words)
 }
 
 size_t tiles_of(int64_t cap) { return (size_t)((cap + qp::kTile - 1) / qp::kTile); }
-
-// Bytes of the append-record stash of `blocks` resident blocks (kStashBufs
-// buffers of kStashFields x kTile doubles each).
-size_t stash_bytes(size_t blocks)
-{
-    return blocks * qp::kStashBufs * (size_t)qp::kStashFieldsHost * qp::kTile * sizeof(double);
-}
 
 // Next free event of the profiling pool (grown on demand).
 cudaError_t next_event(qp_ctx *c, cudaEvent_t *ev)
@@ -696,19 +689,6 @@ int blocks_per_sm(qp_ctx *ctx, int precision, int field_kind, bool batch)
     return bpsm;
 }
 
-// Time of step `step` and the FP32 / double-float time constants of the
-// mixed path (the kernel of a batch computes the same values on the device).
-void set_time_host(qp::Problem &P, int64_t step)
-{
-    P.step = (uint64_t)step;
-    P.t = (double)step * P.dt;
-    const double tr = P.t - P.f.t_focus;
-    P.mc.t_hi = (float)P.t;
-    P.mc.t_lo = (float)(P.t - (double)P.mc.t_hi);
-    P.mc.tr_hi = (float)tr;
-    P.mc.tr_lo = (float)(tr - (double)P.mc.tr_hi);
-}
-
 // Look-back words of a problem's two chains: lepton tiles, photon tiles.
 void chain_words_of(const qp_ctx *ctx, const qp_step_params *s, size_t &lep, size_t &pho)
 {
@@ -735,7 +715,6 @@ int qp_step(qp_ctx *ctx, const qp_step_params *s, void *stream)
     if (st != QP_OK) return st;
     fill_globals(ctx, a);
     a.ctl = ctx->d_ctl;
-    a.n_problems = 0;
     a.problems = nullptr;
     qp::Problem &P = a.single;
     P.lep_words = ctx->d_chain;
@@ -752,19 +731,26 @@ int qp_step(qp_ctx *ctx, const qp_step_params *s, void *stream)
         if (hs[k] != -1) cap_tiles += (int64_t)tiles_of(ctx->species[hs[k]].d.capacity);
     const int64_t resident = (int64_t)bpsm * ctx->num_sms;
     const int grid = (int)(cap_tiles < resident ? (cap_tiles > 0 ? cap_tiles : 1) : resident);
-    if ((size_t)grid > ctx->stash_blocks) {
-        // grows once, to the resident grid (an allocation, synchronous)
+    const bool long_ok = qp::has_long_tiles(s->field.kind) &&
+                         qp::long_tiles(cap_tiles * qp::kWarps, grid);
+    const size_t stash = (size_t)grid * qp::stash_words(long_ok) * sizeof(double);
+    if (stash > ctx->stash_bytes) {
+        // grows (an allocation, synchronous)
         double *p = nullptr;
-        cudaError_t e = cudaMalloc(&p, stash_bytes((size_t)resident));
+        cudaError_t e = cudaMalloc(&p, stash);
         if (e != cudaSuccess) return cuda_status(e);
         cudaFree(ctx->d_stash);
         ctx->d_stash = p;
-        ctx->stash_blocks = (size_t)resident;
+        ctx->stash_bytes = stash;
     }
     a.stash = ctx->d_stash;
     cudaStream_t cs = (cudaStream_t)stream;
-    for (int32_t k = 0; k < s->n_steps; ++k) {
-        set_time_host(P, s->step + k);
+    // several steps a launch; one each while launches are timed
+    const int per = ctx->profiling ? 1 : qp::kStepsPerLaunch;
+    for (int32_t k = 0; k < s->n_steps; k += per) {
+        const int steps = s->n_steps - k < per ? s->n_steps - k : per;
+        P.step = (uint64_t)(s->step + k);
+        a.launch = qp::single_launch(steps, long_ok);
         cudaError_t e = timed(ctx, 0, cs, [&] {
             return qp::launch_step(a, s->precision, s->field.kind, false, grid, cs);
         });
@@ -849,7 +835,9 @@ int qp_batch_create(qp_ctx *ctx, int32_t max_problems, int32_t precision, int32_
     QP_TRY(cudaMemset(b->d_left, 0, n * sizeof(long long)));
     QP_TRY(cudaMalloc(&b->d_pending, 3 * n * sizeof(long long)));
     QP_TRY(cudaMemset(b->d_pending, 0, 3 * n * sizeof(long long)));
-    QP_TRY(cudaMalloc(&b->d_stash, stash_bytes((size_t)b->grid)));
+    QP_TRY(cudaMalloc(&b->d_stash, (size_t)b->grid *
+                                       qp::stash_words(qp::has_long_tiles(field_kind)) *
+                                       sizeof(double)));
     QP_TRY(cudaMalloc(&b->d_work, n * sizeof(long long)));
     QP_TRY(cudaMemset(b->d_work, 0, n * sizeof(long long)));
     QP_TRY(cudaMalloc(&b->d_ctl, sizeof(qp::StepCtl)));
@@ -968,7 +956,7 @@ int qp_batch_step(qp_batch *b, int32_t n_launches, void *stream)
     qp::StepArgs a{};
     fill_globals(b->ctx, a);
     a.ctl = b->d_ctl;
-    a.n_problems = b->max;
+    a.launch = b->max;
     a.problems = b->d_table;
     a.stash = b->d_stash;
     cudaStream_t cs = (cudaStream_t)stream;
@@ -1107,7 +1095,7 @@ int qp_step_fused(qp_ctx *ctx, const qp_step_params *s, int32_t fuse, void *stre
     P.device_step = 0;
     for (int32_t w0 = 0; w0 < s->n_steps; w0 += K) {
         const int Kw = s->n_steps - w0 < K ? s->n_steps - w0 : K;
-        set_time_host(P, s->step + w0);
+        P.step = (uint64_t)(s->step + w0);
         e = timed(ctx, 0, cs, [&] {
             return qp::launch_fused(a, s->precision, s->field.kind, Kw, tiles_e, tiles,
                                     ctx->d_fuse, order_grid, win, ctx->num_sms, cs);

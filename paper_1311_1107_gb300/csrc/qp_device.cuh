@@ -68,8 +68,6 @@ struct TablesDev {
 // Step constants of the mixed path as FP32 values or double-float pairs
 // (split on the host), so the kernel needs no FP64 arithmetic for them.
 struct MixedConsts {
-    float t_hi, t_lo;           // t = n dt
-    float tr_hi, tr_lo;         // t - t_focus (Gaussian pulse)
     float xf_hi, xf_lo;         // x_focus
     float idx_hi, idx_lo, idy_hi, idy_lo;  // 1/dx, 1/dy (Yee grid)
     float x0s_hi, x0s_lo, y0s_hi, y0s_lo;  // x0/dx, y0/dy
@@ -79,6 +77,15 @@ struct MixedConsts {
                                 // that no rounding of the constant biases every chi
     float a0, b0, zr, inv_zr, inv_w0sq, k_env;  // field shape (k_env = 2 ln2 / tau_fwhm^2)
     float nxf, nyf;                            // Yee grid size
+};
+
+// The step being taken: its index and time t = step dt, and the mixed path's
+// constants of it.
+struct StepTime {
+    double t;
+    uint64_t step;
+    float t_hi, t_lo;           // t
+    float tr_hi, tr_lo;         // t - t_focus (Gaussian pulse)
 };
 
 // Device-resident control block of a launch sequence: the tile ticket, the
@@ -92,11 +99,45 @@ struct StepCtl {
 };
 
 constexpr int kMaxProblems = 64;  // problems (independent runs) per launch
-// doubles per thread of one append record (see the stash of qp_step.cuh),
-// and the append-record buffers per block: a tile's appends are written
-// kStashBufs - 1 tiles after its physics
-constexpr int kStashFieldsHost = 7 + 2 * QP_MAX_EMISSIONS;
-constexpr int kStashBufs = 3;
+// doubles of one append record (see the stash of qp_step.cuh), tiles a block
+// has in flight, sub-tiles of 32 slots in a warp's part of a long tile
+constexpr int kStashFieldsHost = 9 + QP_MAX_EMISSIONS;
+constexpr int kStashBufs = 4;
+constexpr int kSubTiles = 8;
+
+// A launch of `subs` sub-tiles of 32 slots on `grid` blocks takes long tiles
+// once every warp has about four of their parts of kSubTiles sub-tiles (below
+// that the last parts leave warps idle), else short ones (see qp_step.cuh).
+constexpr int kPartsPerWarp = 4;
+__host__ __device__ inline bool long_tiles(long long subs, int grid)
+{
+    return subs >= (long long)kSubTiles * kPartsPerWarp * kWarps * grid;
+}
+
+// Steps of a launch of a single problem, and whether its stash has room for
+// long tiles, in one word of the launch parameters (a word more there cost the
+// shortest launches 5 %).
+__host__ __device__ inline int32_t single_launch(int steps, bool long_ok)
+{
+    return steps * 2 + (long_ok ? 1 : 0);
+}
+__host__ __device__ inline int single_steps(int32_t launch) { return launch >> 1; }
+__host__ __device__ inline bool single_long(int32_t launch) { return (launch & 1) != 0; }
+// Steps a launch takes at most: other streams' kernels wait for it.
+constexpr int kStepsPerLaunch = 8;
+
+// Field kinds whose step kernel has the loop over long tiles (see kEmitInPlace).
+__host__ __device__ constexpr bool has_long_tiles(int field_kind)
+{
+    return field_kind != QP_FIELD_YEE2D;
+}
+
+// Doubles of a block's stash: kStashBufs short tiles, or the three parts each
+// warp has in flight of long ones.
+__host__ __device__ inline size_t stash_words(bool long_ok)
+{
+    return (size_t)kStashFieldsHost * kTile * (long_ok ? 3 * kSubTiles : kStashBufs);
+}
 
 // One independent run stepped by a launch: its species, field, step
 // constants, look-back scratch and control words.  A launch steps either a
@@ -105,15 +146,15 @@ constexpr int kStashBufs = 3;
 struct Problem {
     SpeciesDev sp[3];                 // electron, positron, photon
     FieldDev f;
-    MixedConsts mc;                   // t_*, tr_* set per launch on the device
+    MixedConsts mc;
     unsigned long long *lep_words;    // look-back words of the lepton chain
     unsigned long long *pho_words;    // look-back words of the photon chain
     long long *pending;               // [3] new live counts, applied by the last block
     long long *step_ctr;              // device-stepped: next step index
     long long *left_ctr;              // device-stepped: launches still to run (0 = idle)
     long long *work_ctr;              // device-stepped: live slots stepped so far
-    double dt, t;                     // t = step dt, set per launch on the device
-    uint64_t step, seed;
+    double dt;
+    uint64_t step, seed;              // step: the launch's first (a batch: step_ctr)
     double chi_th, gmin;
     int32_t pairs, max_emit;
     int32_t device_step;              // 1: step and activity from step_ctr/left_ctr
@@ -127,9 +168,10 @@ struct StepArgs {
     int *status;                      // sticky status word
     double a_S, C_rate, tau0w;
     unsigned int spin_limit;          // bound of every device-side wait
-    int32_t n_problems;               // 0: the single problem below
-    const Problem *problems;          // device table of n_problems entries
-    double *stash;                    // append records: [block][2][fields][kTile]
+    int32_t launch;                   // batch: problems in the table; single problem: see
+                                      // single_launch
+    const Problem *problems;          // a batch's device table
+    double *stash;                    // append records: stash_words() a block
     Problem single;
 };
 
@@ -196,6 +238,7 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long *bar, unsigned 
 __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, unsigned parity,
                                                   unsigned limit)
 {
+#pragma unroll 1
     for (unsigned k = 0; k < limit; ++k)
         if (mbar_try_wait(bar, parity)) return true;
     return false;

@@ -1,15 +1,15 @@
-// Double-float arithmetic and FP64 <-> double-float conversion by integer
-// operations, for the mixed-precision path.
+// Double-float arithmetic and FP64 <-> double-float conversion for the
+// mixed-precision path.
 //
 // On GB300 every FP64 instruction, and every f32 <-> f64 conversion, issues
 // at about 1/65 of the FP32 rate.  The mixed path therefore keeps the FP64
 // storage of momenta, positions and optical depths, but converts them to
-// double-float pairs (hi + lo, two FP32 numbers, ~47 significant bits) with
-// integer and FP32 instructions only, carries the precision-critical
-// quantities (chi_e's cancellation, the accumulated momentum, position and
-// optical depth) in double-float, and converts back with integer
-// instructions.  Everything here also compiles for the host, where it is
-// tested bit-for-bit against exact double arithmetic.
+// floats or double-float pairs (hi + lo, two FP32 numbers, ~47 significant
+// bits) with integer and FP32 instructions only, carries the
+// precision-critical quantities (chi_e's cancellation, optical depths) in
+// double-float, and spends the FP64 pipe on one addition a component: the
+// new state's (add_fd).  Everything here also compiles for the host, where it
+// is tested against exact arithmetic.
 //
 // The error-free transformations are the classical ones: TwoSum (Knuth),
 // FastTwoSum (Dekker) and TwoProd with a fused multiply-add.
@@ -19,16 +19,11 @@
 
 #ifdef __CUDACC__
 #define QP_HD __host__ __device__ __forceinline__
-// rare cases: called, never inlined, so that the common path's code stays
-// short and carries no predicated-off FP64 instructions
-#define QP_HD_COLD __host__ __device__ inline __noinline__
-// frequent but repeated many times per particle: one called copy keeps the
-// step kernel's instruction footprint small (it measured faster than
-// inlining every call site)
+// repeated many times per particle: one called copy keeps the step kernel's
+// instruction footprint small
 #define QP_HD_SHARED __host__ __device__ inline __noinline__
 #else
 #define QP_HD inline
-#define QP_HD_COLD inline
 #define QP_HD_SHARED inline
 #include <math.h>
 #include <string.h>
@@ -213,23 +208,14 @@ QP_HD df2 split_d(double d)
 {
     const uint64_t b = d2u(d);
     const uint32_t dh = (uint32_t)(b >> 32), dl = (uint32_t)b;
-    const uint32_t e = (dh >> 20) & 0x7FFu;
-    if (e < 897u) return {0.0f, 0.0f};
+    const uint32_t e = (dh >> 20) & 0x7FFu, sign = dh & 0x80000000u;
     // sign | (e - 896) << 23 | top 23 mantissa bits
     const uint32_t top = (dh << 3) | (dl >> 29);
-    const uint32_t hb = ((top - (384u << 23)) & 0x7FFFFFFFu) | (dh & 0x80000000u);
-    // remainder: the low 29 mantissa bits, worth 2^(e - 1075) each
-    const uint32_t r29 = dl & 0x1FFFFFFFu;
-    float lo = 0.0f;
-    if (r29 && e >= 949u) {
-        // exact FP32 values of the two halves, then one rounding in the fma
-        const float fa = u2f(0x4B000000u | (r29 >> 15)) - 8388608.0f;
-        const float fb = u2f(0x4B000000u | (r29 & 0x7FFFu)) - 8388608.0f;
-        const float m = fma32(fa, 32768.0f, fb);
-        lo = m * u2f((e - 948u) << 23);
-        if (dh & 0x80000000u) lo = -lo;
-    }
-    return {u2f(hb), lo};
+    const uint32_t hb = ((top - (384u << 23)) & 0x7FFFFFFFu) | sign;
+    // remainder: the low 29 mantissa bits, worth 2^(e - 1075) each, rounded
+    // to 24 by the conversion
+    const float lo = (float)(dl & 0x1FFFFFFFu) * u2f(((e - 948u) << 23) | sign);
+    return {e < 897u ? 0.0f : u2f(hb), e < 949u ? 0.0f : lo};
 }
 
 // d rounded to the nearest float (ties away from zero) by integer
@@ -258,121 +244,40 @@ QP_HD double f_to_d(float f)
                ((uint64_t)(b & 0x7FFFFFu) << 29));
 }
 
-// hi + lo rounded to double (within one unit in the last place) by integer
-// instructions, for a normalised pair (|lo| <= ulp(hi), as every df2
-// operation above returns).  Pairs outside that range, zero hi, and
-// non-finite values take an FP64 path.
-QP_HD_COLD double merge_df_fp64(float hi, float lo) { return (double)hi + (double)lo; }
+// hi + lo rounded to double.
+QP_HD double merge_df(df2 a) { return f_to_d(a.hi) + f_to_d(a.lo); }
 
-QP_HD double merge_df(df2 a)
+// d + f rounded to double: the FP64 accumulation of an FP32 increment.  The
+// stored double keeps all its bits; only the increment carries FP32 error.
+//   f below 2^29 units of d's last place: one FP64 addition of the exactly
+//     converted f.  The FP64 pipe is nearly idle on this path, and seven
+//     additions a lepton keep it 30 % busy; the same sum by some 25 integer
+//     instructions and a call each took more issue slots than the rest of the
+//     write-back;
+//   larger f, or a sum below a quarter of d: a double-float sum (split_d,
+//     two_sum, one rounded low part), exact to 2^-47 relative.  A momentum
+//     turning through zero, an optical depth near its end and every recoil
+//     are here, so nearly every warp of a step has such lanes: one short
+//     function, called.
+// (Three integer functions calling one another, decoding the operands again
+// each, were 30 % of the 4.2e6-lepton collision step.)
+QP_HD_SHARED double add_fd_wide(double d, float f)
 {
-    const uint32_t hb = f2u(a.hi), lb = f2u(a.lo);
-    const uint32_t eh = (hb >> 23) & 0xFFu, el = (lb >> 23) & 0xFFu;
-    if (eh == 0u || eh == 0xFFu || el == 0xFFu) return merge_df_fp64(a.hi, a.lo);
-    const uint64_t sign = (uint64_t)(hb & 0x80000000u) << 32;
-    int64_t S = (int64_t)((1ull << 52) | ((uint64_t)(hb & 0x7FFFFFu) << 29));
-    if (el != 0u) {
-        // lo in units of 2^-52 of hi's binade: ml * 2^(el - eh + 29)
-        const int k = (int)el - (int)eh + 29;
-        if (k > 8) return merge_df_fp64(a.hi, a.lo);  // not normalised
-        const uint64_t ml = (1ull << 23) | (lb & 0x7FFFFFu);
-        uint64_t L;
-        if (k >= 0)
-            L = ml << k;
-        else if (k > -40)
-            L = (ml + (1ull << (-k - 1))) >> (-k);
-        else
-            L = 0;
-        if ((hb ^ lb) & 0x80000000u)
-            S -= (int64_t)L;
-        else
-            S += (int64_t)L;
-    }
-    uint64_t e = (uint64_t)eh + 896u;
-    if (S >= (int64_t)(1ull << 53)) {
-        S = (S + 1) >> 1;
-        e += 1;
-    } else if (S < (int64_t)(1ull << 52)) {
-        S <<= 1;
-        e -= 1;
-    }
-    return u2d(sign | (e << 52) | ((uint64_t)S & ((1ull << 52) - 1)));
+    const uint32_t ed = (uint32_t)(d2u(d) >> 52) & 0x7FFu, ef = (f2u(f) >> 23) & 0xFFu;
+    if (ed == 0x7FFu || ef == 0xFFu || ed < 897u || ed > 1150u) return d + (double)f;
+    const df2 a = split_d(d);
+    const df2 s = two_sum(a.hi, f);
+    return f_to_d(s.hi) + f_to_d(add_rn(s.lo, a.lo));
 }
 
-// d + f rounded to double (within one unit in the last place) by integer
-// instructions: the FP64 accumulation of an FP32 increment.  The stored
-// double keeps all its bits; only the increment carries FP32 error.
-// add_fd handles the common case inline (d and f normal, f from half a unit
-// of d's last place up to 2^27 units, the sum in d's binade) and calls
-// add_fd_slow for the rest.
-
-// The cases add_fd does not handle in integers (zero or tiny d, increments
-// comparable to or larger than d, large cancellations): through a
-// double-float sum, exact to 2^-47 relative, still without FP64
-// instructions; non-finite values go through FP64.
-QP_HD_COLD double add_fd_wide(double d, float f)
+QP_HD double add_fd(double d, float f)
 {
-    const uint32_t ed = (uint32_t)(d2u(d) >> 52) & 0x7FFu;
-    const uint32_t ef = (f2u(f) >> 23) & 0xFFu;
-    if (ed == 0x7FFu || ef == 0xFFu || (ed != 0u && ed < 897u) || ed > 1150u)
-        return d + (double)f;
-    return merge_df(df_add_f(split_d(d), f));
-}
-
-// The general integer sum (the result may leave d's binade: renormalised,
-// rounded once); zero, non-finite and subnormal operands, increments not
-// much smaller than d, and large cancellations take add_fd_wide.
-QP_HD_COLD double add_fd_slow(double d, float f)
-{
-    const uint32_t fb = f2u(f);
-    if ((fb & 0x7FFFFFFFu) == 0u) return d;
-    const uint64_t db = d2u(d);
-    const uint32_t ed = (uint32_t)(db >> 52) & 0x7FFu, ef = (fb >> 23) & 0xFFu;
-    if (ed == 0u || ed == 0x7FFu || ef == 0u || ef == 0xFFu) return add_fd_wide(d, f);
-    // f in units of d's last place: mf * 2^k, k = ef - ed + 925
+    const uint32_t ed = (uint32_t)(d2u(d) >> 52) & 0x7FFu, ef = (f2u(f) >> 23) & 0xFFu;
+    // f in units of d's last place: (its 24-bit significand) * 2^k
     const int k = (int)ef - (int)ed + 925;
-    if (k > 28) return add_fd_wide(d, f);
-    if (k < -25) return d;  // below half a unit of d
-    const uint64_t mf = (1ull << 23) | (fb & 0x7FFFFFu);
-    const uint64_t L = k >= 0 ? (mf << k) : ((mf + (1ull << (-k - 1))) >> (-k));
-    int64_t S = (int64_t)((1ull << 52) | (db & ((1ull << 52) - 1)));
-    if ((uint32_t)(db >> 63) != (fb >> 31))
-        S -= (int64_t)L;
-    else
-        S += (int64_t)L;
-    uint64_t e = ed;
-    if (S >= (int64_t)(1ull << 53)) {
-        S = (S + 1) >> 1;
-        e += 1;
-    } else if (S < (int64_t)(1ull << 52)) {
-        if (S < (int64_t)(1ull << 51) || e <= 1u) return add_fd_wide(d, f);
-        S <<= 1;
-        e -= 1;
-    }
-    return u2d((db & 0x8000000000000000ull) | (e << 52) | ((uint64_t)S & ((1ull << 52) - 1)));
-}
-
-QP_HD_SHARED double add_fd(double d, float f)
-{
-    const uint32_t fb = f2u(f);
-    if ((fb << 1) == 0u) return d;  // f = +-0
-    const uint64_t db = d2u(d);
-    const uint32_t dh = (uint32_t)(db >> 32);
-    const uint32_t ed = (dh >> 20) & 0x7FFu, ef = (fb >> 23) & 0xFFu;
-    // f in units of d's last place: mf * 2^k, k = ef - ed + 925
-    const int k = (int)ef - (int)ed + 925;
-    if ((ed - 1u) < 0x7FEu && (ef - 1u) < 0xFEu && k <= 27) {
-        if (k < -25) return d;  // below half a unit of d's last place
-        const uint32_t mf = (1u << 23) | (fb & 0x7FFFFFu);
-        // the increment rounded to d's last place (half-way cases away from zero)
-        const uint64_t L =
-            k >= 0 ? ((uint64_t)mf << k) : (uint64_t)((mf + (1u << (-k - 1))) >> (-k));
-        // added to (or taken from) the magnitude bits directly: exact while
-        // the exponent field stays the same, which the test below confirms
-        const uint64_t r = ((dh ^ fb) >> 31) ? db - L : db + L;
-        if (((((uint32_t)(r >> 32)) ^ dh) & 0x7FF00000u) == 0u) return u2d(r);
-    }
-    return add_fd_slow(d, f);
+    const double r = d + f_to_d(f);
+    if (k < 28 || (k == 28 && ((uint32_t)(d2u(r) >> 52) & 0x7FFu) + 1u >= ed)) return r;
+    return add_fd_wide(d, f);
 }
 
 }  // namespace qp

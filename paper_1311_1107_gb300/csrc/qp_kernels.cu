@@ -123,16 +123,16 @@ static const void *step_fn(int precision, int fk, bool batch)
     return precision == QP_MIXED ? step_kernel_mixed(fk, batch) : step_kernel_fp64(fk, batch);
 }
 
-size_t step_smem_bytes(int precision)
+size_t step_smem_bytes(int precision, int field_kind)
 {
-    return precision == QP_MIXED ? step_smem_mixed() : step_smem_fp64();
+    return precision == QP_MIXED ? step_smem_mixed(field_kind) : step_smem_fp64(field_kind);
 }
 
 int step_blocks_per_sm(int precision, int field_kind, bool batch)
 {
     const void *fn = step_fn(precision, field_kind, batch);
     if (!fn) return 1;
-    const size_t smem = step_smem_bytes(precision);
+    const size_t smem = step_smem_bytes(precision, field_kind);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
         return 1;
@@ -147,12 +147,12 @@ cudaError_t launch_step(const StepArgs &a, int precision, int field_kind, bool b
 {
     const void *fn = step_fn(precision, field_kind, batch);
     if (!fn) return cudaErrorInvalidValue;
-    const size_t smem = step_smem_bytes(precision);
+    const size_t smem = step_smem_bytes(precision, field_kind);
     void *args[] = {(void *)&a};
-    // the single-problem mixed-path kernel takes fixed first tiles, which
-    // need every block resident at once: a cooperative launch guarantees it
-    // (or fails to launch)
-    if (!batch && precision == QP_MIXED)
+    // a single problem on the mixed path takes fixed first tiles, and a launch
+    // of several steps meets at their ends: both need every block resident at
+    // once, which a cooperative launch guarantees (or fails to launch)
+    if (!batch && (precision == QP_MIXED || single_steps(a.launch) > 1))
         return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kTile), args, smem, st);
     return cudaLaunchKernel(fn, dim3(grid), dim3(kTile), args, smem, st);
 }

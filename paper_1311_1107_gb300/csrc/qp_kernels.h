@@ -13,9 +13,9 @@ int step_blocks_per_sm(int precision, int field_kind, bool batch);
 // per-precision instantiations of the step kernel (qp_step_fp64.cu, qp_step_mixed.cu)
 const void *step_kernel_fp64(int field_kind, bool batch);
 const void *step_kernel_mixed(int field_kind, bool batch);
-size_t step_smem_fp64();
-size_t step_smem_mixed();
-size_t step_smem_bytes(int precision);
+size_t step_smem_fp64(int field_kind);
+size_t step_smem_mixed(int field_kind);
+size_t step_smem_bytes(int precision, int field_kind);
 // Fused steps (qp_step_fused): one window of K steps of the single problem
 // a.single (its time set for the window's first step).  The physics pass
 // stages each new photon at a provisional index (arrival order) with its

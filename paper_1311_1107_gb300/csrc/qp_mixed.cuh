@@ -1,9 +1,8 @@
 // Mixed-precision particle updates (QP_MIXED): FP32 gather, tables and
-// sampling; chi_e, the Sokolov denominator and the accumulated momentum,
-// position and optical depth carried in double-float (qp_df.h) and written
-// back to the FP64 arrays by integer instructions.  On the common path no
-// instruction uses the FP64 pipe, which issues at ~1/65 of the FP32 rate on
-// GB300.
+// sampling; chi_e, the Sokolov denominator and optical depths carried in
+// double-float (qp_df.h); the FP64 state takes its FP32 increments in one FP64
+// addition each, the only use of the FP64 pipe, which issues at ~1/65 of the
+// FP32 rate on GB300.
 #pragma once
 
 #include "qp_device.cuh"
@@ -27,19 +26,19 @@ __device__ __forceinline__ float reduce_phase(df2 ph)
 // the nearest float elsewhere).
 template <int FK>
 __device__ __forceinline__ void eval_field_mixed(const FieldDev &f, const MixedConsts &m,
-                                                 double xd, double yd, double zd,
+                                                 const StepTime &tm, double xd, double yd, double zd,
                                                  Vec3<float> &E, Vec3<float> &B)
 {
     E = {0.0f, 0.0f, 0.0f};
     B = {0.0f, 0.0f, 0.0f};
     if constexpr (FK == QP_FIELD_PLANE) {
         // E_y = B_z = a0 cos(t - x)
-        const float v = m.a0 * __cosf(reduce_phase(df_sub({m.t_hi, m.t_lo}, split_d(xd))));
+        const float v = m.a0 * __cosf(reduce_phase(df_sub({tm.t_hi, tm.t_lo}, split_d(xd))));
         E.y = v;
         B.z = v;
     } else if constexpr (FK == QP_FIELD_GAUSSIAN) {
         const df2 xi = df_sub(split_d(xd), {m.xf_hi, m.xf_lo});
-        const df2 eta = df_sub({m.tr_hi, m.tr_lo}, xi);  // (t - t_f) - xi
+        const df2 eta = df_sub({tm.tr_hi, tm.tr_lo}, xi);  // (t - t_f) - xi
         const float xf = xi.hi, yf = hi_d(yd), zf = hi_d(zd);
         const float q = xf * m.inv_zr;
         const float wr2 = 1.0f + q * q;
@@ -174,9 +173,11 @@ struct FracPair {
 __device__ __forceinline__ FracPair logit_node(const float *__restrict__ En, int j, float ds,
                                                float t)
 {
-    const float e = __ldg(En + j) * expf(-ds * t);
+    // (products rounded where they stand: the caller's differences would take
+    // them into fused operations)
+    const float e = mul_rn(__ldg(En + j), expf(-ds * t));
     const float x = 1.0f / (1.0f + e);
-    return {x, e * x};
+    return {x, mul_rn(e, x)};
 }
 
 // (a.hi + a.lo) - (c.x + c.y), exact to a rounding of the result
@@ -184,52 +185,77 @@ __device__ __forceinline__ float pair_diff(df2 a, float2 c) { return (a.hi - c.x
 
 __device__ __forceinline__ float2 ldg2(const float2 *p) { return __ldg(p); }
 
-// Invert one row at xi (eta = 1 - xi, from the same random bits): the lower
-// half searches the row C for xi, the upper half searches its complement
+// The inversion of one row at xi (eta = 1 - xi, from the same random bits):
+// the lower half searches the row C for xi, the upper half its complement
 // Q = 1 - C for eta.  Rows, xi and eta are float pairs, so the position
 // between two nodes, (xi - C_j)/(C_j+1 - C_j), keeps FP32 relative precision
 // even where neighbouring nodes differ by 1e-3 or less.
-__device__ __forceinline__ FracPair row_invert_f(const float2 *__restrict__ C,
-                                                 const float2 *__restrict__ Q,
-                                                 const unsigned char *__restrict__ guide,
-                                                 const float *__restrict__ En, df2 xi, df2 eta,
+// The interval is the last node below the key: the guide entry, then a
+// forward scan of mostly none to two nodes.  An emission round is a chain of
+// dependent loads that nothing hides when a problem fills the GPU once, so
+// the entry's next four nodes are loaded together (RowWindow, both rows of a
+// sample before either is used): two round trips a sample, where a node at a
+// time of one row after the other took about ten (2D foil: 90 % of the warps
+// through their first tile's events after 24 us of a step).
+struct RowWindow {
+    float2 edge;   // C_0 of the lower half, Q_last of the upper
+    float2 w[4];   // nodes g .. g + 3 (up to the last)
+    int g;
+};
+
+// sign of the scan's condition: the key is still past node v
+__device__ __forceinline__ bool key_past(bool lower, df2 key, float2 v)
+{
+    const float d = pair_diff(key, v);
+    return lower ? d > 0.0f : d < 0.0f;
+}
+
+__device__ __forceinline__ FracPair row_invert_f(const RowWindow &r, const float2 *__restrict__ V,
+                                                 const float *__restrict__ En, bool lower, df2 key,
                                                  float ds, bool power_tail)
 {
-    if (xi.hi <= 0.5f) {
-        const float2 c0 = ldg2(C);
-        if (pair_diff(xi, c0) <= 0.0f) {
-            const FracPair p0 = logit_node(En, 0, ds, 0.0f);
-            if (power_tail && c0.x > 0.0f) {
-                // below the first node u grows as xi^3 (the u^(1/3) law)
-                const float r = (xi.hi + xi.lo) / (c0.x + c0.y);
-                const float x = p0.x * r * r * r;
-                return {x, 1.0f - x};
+    int lo = r.g;
+    float2 c_lo = r.w[0], c_hi = r.w[1];
+    if (lo < kNNode - 2 && key_past(lower, key, c_hi)) {
+        ++lo;
+        c_lo = c_hi;
+        c_hi = r.w[2];
+        if (lo < kNNode - 2 && key_past(lower, key, c_hi)) {
+            ++lo;
+            c_lo = c_hi;
+            c_hi = r.w[3];
+#pragma unroll 1
+            while (lo < kNNode - 2 && key_past(lower, key, c_hi)) {
+                ++lo;
+                c_lo = c_hi;
+                c_hi = ldg2(V + lo + 1);
             }
-            return p0;
         }
-        // the last node below xi: guide entry, then a forward scan
-        int lo = (int)__ldg(guide + guide_bucket(xi.hi));
-#pragma unroll 1
-        while (lo < kNNode - 2 && pair_diff(xi, ldg2(C + lo + 1)) > 0.0f) ++lo;
-        const float2 c_lo = ldg2(C + lo), c_hi = ldg2(C + lo + 1);
-        const float den = (c_hi.x - c_lo.x) + (c_hi.y - c_lo.y);
-        const float t = den > 0.0f ? fminf(pair_diff(xi, c_lo) / den, 1.0f) : 0.0f;
-        return logit_node(En, lo, ds, t);
     }
-    if (pair_diff(eta, ldg2(Q + kNNode - 1)) <= 0.0f) return logit_node(En, kNNode - 1, ds, 0.0f);
-    // Q decreases along the row: the last node with Q > eta (guide, then scan)
-    int lo = (int)__ldg(guide + kNCdf * kGuideBuckets + guide_bucket(eta.hi));
-#pragma unroll 1
-    while (lo < kNNode - 2 && pair_diff(eta, ldg2(Q + lo + 1)) < 0.0f) ++lo;
-    const float2 q_lo = ldg2(Q + lo), q_hi = ldg2(Q + lo + 1);
-    const float den = (q_lo.x - q_hi.x) + (q_lo.y - q_hi.y);
-    const float t = den > 0.0f ? fminf(-pair_diff(eta, q_lo) / den, 1.0f) : 0.0f;
-    return logit_node(En, lo, ds, fmaxf(t, 0.0f));
+    float t = 0.0f;
+    bool below = false;
+    if (pair_diff(key, r.edge) <= 0.0f) {
+        // past the table's end
+        lo = lower ? 0 : kNNode - 1;
+        below = lower && power_tail && r.edge.x > 0.0f;
+    } else if (lower) {
+        const float den = (c_hi.x - c_lo.x) + (c_hi.y - c_lo.y);
+        t = den > 0.0f ? fminf(pair_diff(key, c_lo) / den, 1.0f) : 0.0f;
+    } else {
+        const float den = (c_lo.x - c_hi.x) + (c_lo.y - c_hi.y);
+        t = den > 0.0f ? fminf(-pair_diff(key, c_lo) / den, 1.0f) : 0.0f;
+        t = fmaxf(t, 0.0f);
+    }
+    const FracPair p = logit_node(En, lo, ds, t);
+    if (!below) return p;
+    // below the first node u grows as xi^3 (the u^(1/3) law)
+    const float q = (key.hi + key.lo) / (r.edge.x + r.edge.y);
+    const float x = mul_rn(p.x * q * q, q);
+    return {x, sub_rn(1.0f, x)};
 }
 
 // Inverse CDF of Eq. 7 (emission rows) or of the pair spectrum, linear
-// between the two chi rows around chi (same rule as the FP64 path).  One
-// copy of the row inversion serves both rows (a loop of one or two).
+// between the two chi rows around chi (same rule as the FP64 path).
 __device__ __forceinline__ FracPair sample_cdf_f(const float2 *__restrict__ rows,
                                                  const float2 *__restrict__ qrows,
                                                  const unsigned char *__restrict__ guide,
@@ -248,17 +274,28 @@ __device__ __forceinline__ FracPair sample_cdf_f(const float2 *__restrict__ rows
         j = grid_index32<2>(chi, f);
         nrow = 2;
     }
-    FracPair a{0.0f, 1.0f}, b{0.0f, 1.0f};
-#pragma unroll 1
-    for (int k = 0; k < nrow; ++k, ++j) {
-        const FracPair r = row_invert_f(rows + j * kNNode, qrows + j * kNNode,
-                                        guide + j * kGuideBuckets, En, xi, eta, ds, emission);
-        if (k == 0)
-            a = r;
-        else
-            b = r;
+    const bool lower = xi.hi <= 0.5f;
+    const df2 key = lower ? xi : eta;
+    const float2 *V = (lower ? rows : qrows) + j * kNNode;
+    const unsigned char *gd = guide + (lower ? 0 : kNCdf * kGuideBuckets) + j * kGuideBuckets +
+                              guide_bucket(key.hi);
+    // a single row is read as both of a pair
+    const int dn = nrow == 2 ? kNNode : 0, dg = nrow == 2 ? kGuideBuckets : 0;
+    RowWindow r[2];
+    r[0].g = (int)__ldg(gd);
+    r[1].g = (int)__ldg(gd + dg);
+    r[0].edge = ldg2(V + (lower ? 0 : kNNode - 1));
+    r[1].edge = ldg2(V + dn + (lower ? 0 : kNNode - 1));
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            r[k].w[i] = ldg2(V + k * dn + min(r[k].g + i, kNNode - 1));
+    const FracPair a = row_invert_f(r[0], V, En, lower, key, ds, emission);
+    if (nrow == 2) {
+        const FracPair b = row_invert_f(r[1], V + dn, En, lower, key, ds, emission);
+        return {a.x + f * (b.x - a.x), a.omx + f * (b.omx - a.omx)};
     }
-    if (nrow == 2) return {a.x + f * (b.x - a.x), a.omx + f * (b.omx - a.omx)};
     if (below && emission) {
         const float x = (chi / (float)kChiLo) * a.x;
         return {x, 1.0f - x};

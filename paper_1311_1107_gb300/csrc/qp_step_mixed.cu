@@ -10,7 +10,7 @@ const void *step_kernel_mixed(int field_kind, bool batch)
     return batch ? step_kernel_of<kMixed, true>(field_kind) : step_kernel_of<kMixed, false>(field_kind);
 }
 
-size_t step_smem_mixed() { return sizeof(Smem<float>); }
+size_t step_smem_mixed(int field_kind) { return step_smem_of<float>(field_kind); }
 
 const void *fused_kernel_mixed(int field_kind) { return fused_kernel_of<kMixed>(field_kind); }
 const void *fused_photons_mixed() { return (const void *)k_fused_photons<kMixed>; }
