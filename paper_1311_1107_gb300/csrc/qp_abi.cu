@@ -601,10 +601,10 @@ int build_problem(const qp_ctx *ctx, const qp_step_params *s, qp::Problem &P)
     P.f.x0 = f.x0;
     P.f.y0 = f.y0;
     if (f.kind == QP_FIELD_YEE2D) {
-        P.f.inv_dx = 1.0 / f.dx;
-        P.f.inv_dy = 1.0 / f.dy;
-        P.f.x0s = f.x0 / f.dx;
-        P.f.y0s = f.y0 / f.dy;
+        P.f.c[0] = 1.0 / f.dx;
+        P.f.c[1] = 1.0 / f.dy;
+        P.f.c[2] = f.x0 / f.dx;
+        P.f.c[3] = f.y0 / f.dy;
     }
     P.dt = s->dt;
     P.step = (uint64_t)s->step;
@@ -620,14 +620,14 @@ int build_problem(const qp_ctx *ctx, const qp_step_params *s, qp::Problem &P)
     m.xf_hi = hi_of(f.x_focus);
     m.xf_lo = lo_of(f.x_focus);
     if (f.kind == QP_FIELD_YEE2D) {
-        m.idx_hi = hi_of(P.f.inv_dx);
-        m.idx_lo = lo_of(P.f.inv_dx);
-        m.idy_hi = hi_of(P.f.inv_dy);
-        m.idy_lo = lo_of(P.f.inv_dy);
-        m.x0s_hi = hi_of(P.f.x0s);
-        m.x0s_lo = lo_of(P.f.x0s);
-        m.y0s_hi = hi_of(P.f.y0s);
-        m.y0s_lo = lo_of(P.f.y0s);
+        m.idx_hi = hi_of(P.f.c[0]);
+        m.idx_lo = lo_of(P.f.c[0]);
+        m.idy_hi = hi_of(P.f.c[1]);
+        m.idy_lo = lo_of(P.f.c[1]);
+        m.x0s_hi = hi_of(P.f.c[2]);
+        m.x0s_lo = lo_of(P.f.c[2]);
+        m.y0s_hi = hi_of(P.f.c[3]);
+        m.y0s_lo = lo_of(P.f.c[3]);
         m.nxf = (float)f.nx;
         m.nyf = (float)f.ny;
     }
@@ -644,6 +644,10 @@ int build_problem(const qp_ctx *ctx, const qp_step_params *s, qp::Problem &P)
     m.b0 = (float)f.b0;
     if (f.kind == QP_FIELD_GAUSSIAN) {
         const double zr = 0.5 * f.w0 * f.w0;
+        P.f.c[0] = 1.0 / zr;
+        P.f.c[1] = 1.0 / (f.w0 * f.w0);
+        P.f.c[2] = 2.0 * 0.6931471805599453 / (f.tau_fwhm * f.tau_fwhm);
+        P.f.c[3] = 0.5 / (zr * zr);
         m.zr = (float)zr;
         m.inv_zr = (float)(1.0 / zr);
         m.inv_w0sq = (float)(1.0 / (f.w0 * f.w0));
@@ -675,7 +679,7 @@ void fill_globals(const qp_ctx *ctx, qp::StepArgs &a)
     a.tab.Gp = ctx->d_guide + 2 * kGuideHalf;
     a.stats = ctx->d_stats;
     a.status = ctx->d_status;
-    a.a_S = ctx->U.a_S;
+    a.inv_aS = 1.0 / ctx->U.a_S;
     a.C_rate = ctx->U.C_rate;
     a.tau0w = ctx->U.tau0w;
     a.spin_limit = kSpinLimit;

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "qp_df.h"
 #include "qp_internal.h"
 
 namespace qp {
@@ -52,7 +53,9 @@ struct FieldDev {
     const float *yee[6];
     int64_t nx, ny;
     double dx, dy, x0, y0;
-    double inv_dx, inv_dy, x0s, y0s;  // 1/dx, 1/dy, x0/dx, y0/dy (mixed gather)
+    // YEE2D: 1/dx, 1/dy, x0/dx, y0/dy; GAUSSIAN, with zr = w0^2/2: 1/zr, 1/w0^2,
+    // 2 ln2 / tau_fwhm^2, 1/(2 zr^2)
+    double c[4];
 };
 
 struct TablesDev {
@@ -166,7 +169,7 @@ struct StepArgs {
     StepCtl *ctl;
     DevStats *stats;                  // counters, indexed by species handle
     int *status;                      // sticky status word
-    double a_S, C_rate, tau0w;
+    double inv_aS, C_rate, tau0w;     // 1/a_S
     unsigned int spin_limit;          // bound of every device-side wait
     int32_t launch;                   // batch: problems in the table; single problem: see
                                       // single_launch
@@ -284,6 +287,53 @@ __device__ __forceinline__ double u53(unsigned a, unsigned b)
     return (double)(m + 1ull) * 0x1.0p-53;
 }
 
+// ------------------------------------------------------------------ FP64 roots and reciprocals
+
+// The FP64 pipe issues one warp instruction in about 20 cycles of an SM, so
+// the FP64 path is bound by their number.  An IEEE square root or division
+// takes about ten; here a Newton iteration of third order (Householder's
+// method) from an FP32 seed takes three for a reciprocal and nine for a root
+// with its reciprocal, the conversions of the seed being integer
+// instructions.  Results are within one unit of the last place.  Arguments
+// outside FP32's range go to the IEEE operations.  (With the gather's integer
+// conversions and one sampling copy for both CDF rows: 2D foil 209 -> 119 us a
+// step of 131072 e-, the 2e5-electron collision 316 -> 205 us.)
+
+__device__ __forceinline__ bool in_fp32_range(double x)
+{
+    const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7FFu;
+    return e - 903u <= 1143u - 903u;  // 2^-120 <= |x| < 2^121
+}
+
+static __device__ __noinline__ double rcp64_ieee(double x) { return 1.0 / x; }
+
+__device__ __forceinline__ double rcp64(double x)
+{
+    if (!in_fp32_range(x)) return rcp64_ieee(x);
+    const double y = f_to_d(__fdividef(1.0f, hi_d(x)));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// 1/sqrt(x) for x > 0.
+static __device__ __noinline__ double rsqrt64_ieee(double x) { return 1.0 / sqrt(x); }
+
+__device__ __forceinline__ double rsqrt64(double x)
+{
+    if (!in_fp32_range(x)) return rsqrt64_ieee(x);
+    const double y = f_to_d(rsqrtf(hi_d(x)));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+// sqrt(x) from r = 1/sqrt(x) (x >= 0; 0 and infinity pass through).
+__device__ __forceinline__ double root_of(double x, double r)
+{
+    if (!in_fp32_range(x)) return sqrt(x);
+    const double s = x * r;
+    return fma(fma(-s, s, x), 0.5 * r, s);
+}
+
 // ------------------------------------------------------------------ fields
 
 template <typename R>
@@ -331,6 +381,17 @@ __device__ __forceinline__ R yee_interp(const float *__restrict__ F, const YeeSt
     return acc;
 }
 
+// A node's value in the gather's type; to FP64 by integer instructions (the
+// conversion unit is the FP64 pipe).
+template <typename R>
+__device__ __forceinline__ R node_value(float v)
+{
+    if constexpr (sizeof(R) == 8)
+        return f_to_d(v);
+    else
+        return v;
+}
+
 template <typename R>
 __device__ __forceinline__ void yee_gather(const FieldDev &f, const int ix[2], const int iy[2],
                                            const R wx[2], const R wy[2], Vec3<R> &E, Vec3<R> &B)
@@ -369,13 +430,21 @@ __device__ __forceinline__ void yee_gather(const FieldDev &f, const int ix[2], c
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             const YeeStencil<R> &q = st[comp_st[c]];
+            if constexpr (sizeof(R) == 8) {
+                // a component that is zero around the particle (four of a
+                // wave's six, for a whole warp) costs no FP64 instruction
+                const unsigned any = __float_as_uint(v[c][0]) | __float_as_uint(v[c][1]) |
+                                     __float_as_uint(v[c][2]) | __float_as_uint(v[c][3]);
+                out[c] = R(0);
+                if ((any << 1) == 0u) continue;
+            }
             const R w00 = (R(1) - q.wx) * (R(1) - q.wy), w10 = q.wx * (R(1) - q.wy);
             const R w01 = (R(1) - q.wx) * q.wy, w11 = q.wx * q.wy;
             R acc = R(0);
-            acc += w00 * (R)v[c][0];
-            acc += w10 * (R)v[c][1];
-            acc += w01 * (R)v[c][2];
-            acc += w11 * (R)v[c][3];
+            acc += w00 * node_value<R>(v[c][0]);
+            acc += w10 * node_value<R>(v[c][1]);
+            acc += w01 * node_value<R>(v[c][2]);
+            acc += w11 * node_value<R>(v[c][3]);
             out[c] = acc;
         }
         E = {out[0], out[1], out[2]};
@@ -390,72 +459,63 @@ __device__ __forceinline__ void yee_gather(const FieldDev &f, const int ix[2], c
     B.z = yee_interp<R>(f.yee[5], st[3], nx, ny);
 }
 
-// Fields at (x, y, z, t); R = double (FP64 path) or float (mixed path, with
-// phases reduced in FP64 before the FP32 trigonometry).
-template <int FK, typename R>
-__device__ __forceinline__ void eval_field(const FieldDev &f, double x, double y, double z,
-                                           double t, Vec3<R> &E, Vec3<R> &B)
+// a / b rounded to nearest, from r = 1/b rounded to nearest (Markstein's
+// correction): the last bit of a cell coordinate of a thousand is 1e-13 of a
+// weight, far above the rounding of anything else in a step.
+__device__ __forceinline__ double quotient64(double a, double b, double r)
 {
-    E = {R(0), R(0), R(0)};
-    B = {R(0), R(0), R(0)};
+    const double q = a * r;
+    return fma(fma(-q, b, a), r, q);
+}
+
+// The cell index i of a coordinate a and its weight a - i, for the node grid
+// (h = 0) and the half-node grid (h = 1, floor(a - 1/2)); i clamped to
+// -2 .. n + 1, NaN to n + 1 (outside: no field).
+__device__ __forceinline__ void cell64(double a, int n, int i[2], double w[2])
+{
+    const double f = floor(a);
+    const bool nan = (__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFll) > 0x7FF0000000000000ll;
+    const int c = nan ? n + 1 : __double2int_rz(f);  // saturates
+    w[0] = a - f;
+    const bool upper = __double2hiint(w[0]) >= 0x3FE00000;  // w >= 1/2
+    w[1] = w[0] + (upper ? -0.5 : 0.5);  // exact
+    i[0] = max(-2, min(n + 1, c));
+    i[1] = max(-2, min(n + 1, nan ? n + 1 : upper ? c : max(c, -2) - 1));
+}
+
+// Fields of the FP64 path at (x, y, z, t).
+template <int FK>
+__device__ __forceinline__ void eval_field(const FieldDev &f, double x, double y, double z,
+                                           double t, Vec3<double> &E, Vec3<double> &B)
+{
+    E = {0.0, 0.0, 0.0};
+    B = {0.0, 0.0, 0.0};
     if constexpr (FK == QP_FIELD_PLANE) {
-        R v;
-        if constexpr (sizeof(R) == 8) {
-            v = f.a0 * cos(t - x);
-        } else {
-            const double ph = t - x;
-            const double red = ph - 6.283185307179586 * rint(ph * 0.15915494309189535);
-            v = (float)f.a0 * cosf((float)red);
-        }
+        const double v = f.a0 * cos(t - x);
         E.y = v;
         B.z = v;
     } else if constexpr (FK == QP_FIELD_GAUSSIAN) {
         const double xi = x - f.x_focus;
         const double eta = (t - f.t_focus) - xi;
-        const double zr = 0.5 * f.w0 * f.w0;
-        const double q = xi / zr;
-        const double wr2 = 1.0 + q * q;
-        const double r2 = y * y + z * z;
-        R v;
-        if constexpr (sizeof(R) == 8) {
-            const double env = -r2 / (f.w0 * f.w0 * wr2) -
-                               2.0 * 0.6931471805599453 * eta * eta / (f.tau_fwhm * f.tau_fwhm);
-            const double amp = f.a0 / sqrt(wr2) * exp(env);
-            const double phase = -eta + r2 * xi / (2.0 * (xi * xi + zr * zr)) - atan(q);
-            v = amp * cos(phase);
-        } else {
-            const float env = (float)(-r2 / (f.w0 * f.w0 * wr2)) -
-                              1.3862943611198906f * (float)(eta * eta / (f.tau_fwhm * f.tau_fwhm));
-            const float amp = (float)f.a0 * rsqrtf((float)wr2) * __expf(env);
-            double phase = -eta + r2 * xi / (2.0 * (xi * xi + zr * zr));
-            phase -= 6.283185307179586 * rint(phase * 0.15915494309189535);
-            v = amp * cosf((float)phase - atanf((float)q));
-        }
+        const double q = xi * f.c[0];
+        const double ir = rsqrt64(1.0 + q * q), iwr2 = ir * ir;  // 1/sqrt(1 + q^2)
+        const double r2w = (y * y + z * z) * iwr2;
+        const double env = -r2w * f.c[1] - f.c[2] * eta * eta;
+        const double phase = -eta + r2w * xi * f.c[3] - atan(q);
+        const double v = f.a0 * ir * exp(env) * cos(phase);
         E.y = v;
         B.z = v;
     } else if constexpr (FK == QP_FIELD_UNIFORM_B) {
-        B.z = (R)f.b0;
+        B.z = f.b0;
     } else if constexpr (FK == QP_FIELD_YEE2D) {
         // linear interpolation of the six staggered components
         //   Ex(i+1/2,j) Ey(i,j+1/2) Ez(i,j) Bx(i,j+1/2) By(i+1/2,j) Bz(i+1/2,j+1/2);
-        // nodes outside the grid contribute zero field.  The cell index and
-        // weight of each axis are found once for the node and the half-node
-        // grids (FP64 path: in FP64; mixed path: the cell coordinate is formed
-        // with one FP64 FMA, the rest in FP32).
+        // nodes outside the grid contribute zero field
         int ix[2], iy[2];
-        R wx[2], wy[2];
-        const double gx = (x - f.x0) / f.dx, gy = (y - f.y0) / f.dy;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const double ax = h ? gx - 0.5 : gx, ay = h ? gy - 0.5 : gy;
-            const double fx = floor(ax), fy = floor(ay);
-            wx[h] = (R)(ax - fx);
-            wy[h] = (R)(ay - fy);
-            // clamp before the conversion (NaN and huge values included)
-            ix[h] = (int)fmax(-2.0, fmin((double)f.nx + 1.0, fx));
-            iy[h] = (int)fmax(-2.0, fmin((double)f.ny + 1.0, fy));
-        }
-        yee_gather<R>(f, ix, iy, wx, wy, E, B);
+        double wx[2], wy[2];
+        cell64(quotient64(x - f.x0, f.dx, f.c[0]), (int)f.nx, ix, wx);
+        cell64(quotient64(y - f.y0, f.dy, f.c[1]), (int)f.ny, iy, wy);
+        yee_gather<double>(f, ix, iy, wx, wy, E, B);
     }
 }
 
@@ -464,14 +524,14 @@ __device__ __forceinline__ void eval_field(const FieldDev &f, double x, double y
 // chi_e = sqrt(|gamma E + u x B|^2 - (u.E)^2) / a_S, in FP64
 __device__ __forceinline__ double chi_e64(double Ex, double Ey, double Ez, double Bx, double By,
                                           double Bz, double ux, double uy, double uz, double g,
-                                          double a_S)
+                                          double inv_aS)
 {
     const double ax = g * Ex + (uy * Bz - uz * By);
     const double ay = g * Ey + (uz * Bx - ux * Bz);
     const double az = g * Ez + (ux * By - uy * Bx);
     const double ue = ux * Ex + uy * Ey + uz * Ez;
     const double s = ax * ax + ay * ay + az * az - ue * ue;
-    return s > 0.0 ? sqrt(s) / a_S : 0.0;
+    return s > 0.0 ? root_of(s, rsqrt64(s)) * inv_aS : 0.0;
 }
 
 // ------------------------------------------------------------------ rate tables
@@ -486,7 +546,9 @@ __device__ __forceinline__ int grid_index64(double chi, double &f)
     const unsigned long long b = (unsigned long long)__double_as_longlong(chi);
     const int e = (int)((b >> 52) & 0x7FF) - 1023;
     const int m = (int)((b >> (52 - KBITS)) & ((1u << KBITS) - 1));
-    f = (double)(b & ((1ull << (52 - KBITS)) - 1)) * (1.0 / (double)(1ull << (52 - KBITS)));
+    // the rest of the mantissa, as 1.rest - 1
+    const unsigned long long rest = (b << KBITS) & ((1ull << 52) - 1);
+    f = __longlong_as_double((long long)((1023ull << 52) | rest)) - 1.0;
     return ((e - kChiExp0) << KBITS) + m;
 }
 
@@ -511,7 +573,7 @@ __device__ __forceinline__ double rate64(const double *V, double chi, bool &clam
     if (WHICH == 2 && !(chi >= kPairChiMin)) return 0.0;
     if (!(chi >= kChiLo)) {
         if (WHICH == 0) return __dmul_rn(2.5 * kPi, chi);
-        return __dmul_rn(__dmul_rn(2.0 * kPi, chi), chi) / 1.7320508075688772;
+        return __dmul_rn(__dmul_rn(2.0 * kPi / 1.7320508075688772, chi), chi);
     }
     double v, c = chi;
     if (chi >= kChiHi) {
@@ -525,7 +587,7 @@ __device__ __forceinline__ double rate64(const double *V, double chi, bool &clam
         v = __dadd_rn(a, __dmul_rn(f, d));
     }
     if (WHICH == 1) return __dmul_rn(v, c);
-    if (WHICH == 2) return __dmul_rn(v, exp(-8.0 / (3.0 * c)));
+    if (WHICH == 2) return __dmul_rn(v, exp(-8.0 / 3.0 * rcp64(c)));
     return v;
 }
 
@@ -582,70 +644,63 @@ __device__ __forceinline__ int guide_bucket(float x)
     return min(max(m, 0), kGuideBuckets - 1);
 }
 
-// Invert one CDF row C (kNNode logit nodes s_i = smin + span i / 255) at xi.
+// Invert one CDF row C (kNNode logit nodes s_i = smin + ds i) at xi, in FP64.
 // Emission rows follow u^(1/3) below the first node; pair rows clamp.
-template <typename R>
-__device__ __forceinline__ R row_invert(const R *__restrict__ C,
-                                        const unsigned char *__restrict__ guide, R xi,
-                                        double smin, double span, bool power_tail)
+__device__ __forceinline__ double row_invert(const double *__restrict__ C,
+                                             const unsigned char *__restrict__ guide, double xi,
+                                             double smin, double ds, bool power_tail)
 {
-    const R c0 = __ldg(C);
+    const double c0 = __ldg(C);
+    // the last node below xi: guide entry, then a forward scan (past the ends:
+    // the first or the last node)
+    double pos = 0.0, tail = 1.0;
     if (xi <= c0) {
-        const R x0 = R(1) / (R(1) + (R)exp(-smin));
-        if (power_tail && c0 > R(0)) {
-            const R r = xi / c0;
-            return x0 * r * r * r;
+        if (power_tail && c0 > 0.0) {
+            const double r = xi * rcp64(c0);
+            tail = r * r * r;
         }
-        return x0;
-    }
-    const R clast = __ldg(C + kNNode - 1);
-    if (xi >= clast) return R(1) / (R(1) + (R)exp(-(smin + span)));
-    // the last node below xi: guide entry, then a forward scan
-    int lo = xi <= R(0.5) ? (int)__ldg(guide + guide_bucket(xi))
-                          : (int)__ldg(guide + kNCdf * kGuideBuckets + guide_bucket(R(1) - xi));
-#pragma unroll 1
-    while (lo < kNNode - 2 && __ldg(C + lo + 1) < xi) ++lo;
-    const R clo = __ldg(C + lo), chi_ = __ldg(C + lo + 1);
-    const double s_lo = smin + span * lo / (kNNode - 1);
-    const double s_hi = smin + span * (lo + 1) / (kNNode - 1);
-    if constexpr (sizeof(R) == 8) {
-        const double t = (xi - clo) / (chi_ - clo);
-        const double sv = s_lo + t * (s_hi - s_lo);
-        return 1.0 / (1.0 + exp(-sv));
+    } else if (xi >= __ldg(C + kNNode - 1)) {
+        pos = (double)(kNNode - 1);
     } else {
-        const float t = (xi - clo) / (chi_ - clo);
-        const float sv = (float)s_lo + t * (float)(s_hi - s_lo);
-        return 1.0f / (1.0f + __expf(-sv));
+        int lo = xi <= 0.5 ? (int)__ldg(guide + guide_bucket(xi))
+                           : (int)__ldg(guide + kNCdf * kGuideBuckets + guide_bucket(1.0 - xi));
+#pragma unroll 1
+        while (lo < kNNode - 2 && __ldg(C + lo + 1) < xi) ++lo;
+        const double clo = __ldg(C + lo), chi_ = __ldg(C + lo + 1);
+        pos = (double)lo + (xi - clo) * rcp64(chi_ - clo);
     }
+    return tail * rcp64(1.0 + exp(-fma(ds, pos, smin)));
 }
 
 // Photon fraction u = chi_gamma / chi_e for chi_e (rows j, j+1 interpolated
-// linearly in chi; below the grid the classical scaling u ~ chi).
-template <typename R>
-__device__ __forceinline__ R sample_cdf(const R *__restrict__ rows,
-                                        const unsigned char *__restrict__ guide, R chi, R xi,
-                                        double smin, double span, bool emission, bool &clamped)
+// linearly in chi; below the grid the classical scaling u ~ chi).  One copy of
+// the row inversion serves both rows.
+__device__ __forceinline__ double sample_cdf(const double *__restrict__ rows,
+                                             const unsigned char *__restrict__ guide, double chi,
+                                             double xi, double smin, double span, bool emission,
+                                             bool &clamped)
 {
-    if (!(chi >= (R)kChiLo)) {
-        const R r0 = row_invert<R>(rows, guide, xi, smin, span, emission);
-        return emission ? (chi / (R)kChiLo) * r0 : r0;
+    const double ds = span / (kNNode - 1);
+    const bool below = !(chi >= kChiLo);
+    double f = 0.0;
+    int j = 0, nrow = 1;
+    if (!below) {
+        if (chi >= kChiHi) {
+            clamped = true;
+            j = kNCdf - 1;
+        } else {
+            j = grid_index64<2>(chi, f);
+            nrow = 2;
+        }
     }
-    if (chi >= (R)kChiHi) {
-        clamped = true;
-        return row_invert<R>(rows + (kNCdf - 1) * kNNode, guide + (kNCdf - 1) * kGuideBuckets,
-                             xi, smin, span, emission);
+    double a = 0.0, b = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < nrow; ++k, ++j) {
+        b = row_invert(rows + j * kNNode, guide + j * kGuideBuckets, xi, smin, ds, emission);
+        if (k == 0) a = b;
     }
-    R f;
-    int j;
-    if constexpr (sizeof(R) == 8)
-        j = grid_index64<2>(chi, f);
-    else
-        j = grid_index32<2>(chi, f);
-    const R ra = row_invert<R>(rows + j * kNNode, guide + j * kGuideBuckets, xi, smin, span,
-                               emission);
-    const R rb = row_invert<R>(rows + (j + 1) * kNNode, guide + (j + 1) * kGuideBuckets, xi,
-                               smin, span, emission);
-    return ra + f * (rb - ra);
+    if (nrow == 2) return a + f * (b - a);
+    return below && emission ? chi * (1.0 / kChiLo) * a : a;
 }
 
 // ------------------------------------------------------------------ FP32 inverse CDF with complement

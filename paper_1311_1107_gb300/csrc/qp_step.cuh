@@ -249,7 +249,8 @@ constexpr int kQueue = 64;
 // What a lepton carries out of its push: momentum after it (mixed path: the
 // FP32 increment of the FP64 momentum), gamma, chi_e, W dt and the fields; a lepton
 // without an event needs no fields any more: E holds delta v, chi the
-// decrement of its optical depth (FP64: the new one) and B the FP32 momentum.
+// decrement of its optical depth (FP64: the new one), gam 1/gamma in FP64 and B
+// the FP32 momentum.
 template <typename R>
 struct LeptonMid {
     R ux, uy, uz, gam, chi, wdt;
@@ -408,51 +409,52 @@ __device__ __forceinline__ bool lepton_push(const StepArgs &a, const Problem &P,
         double ux = s.ux, uy = s.uy, uz = s.uz;
         double tau = s.tau;
         Vec3<R> E, B;
-        eval_field<FK, R>(P.f, x0, y0, z0, tm.t, E, B);
+        eval_field<FK>(P.f, x0, y0, z0, tm.t, E, B);
 
         // ---- Boris push of the Lorentz force (f_l of Eq. 4)
         {
             const double h = 0.5 * q * dt;
             const double mx = ux + h * E.x, my = uy + h * E.y, mz = uz + h * E.z;
-            const double g = sqrt(1.0 + mx * mx + my * my + mz * mz);
-            const double tx = h * B.x / g, ty = h * B.y / g, tz = h * B.z / g;
-            const double t2 = tx * tx + ty * ty + tz * tz;
-            const double sx = 2.0 * tx / (1.0 + t2), sy = 2.0 * ty / (1.0 + t2),
-                         sz = 2.0 * tz / (1.0 + t2);
+            const double hig = h * rsqrt64(1.0 + mx * mx + my * my + mz * mz);
+            const double tx = hig * B.x, ty = hig * B.y, tz = hig * B.z;
+            const double k2 = 2.0 * rcp64(1.0 + tx * tx + ty * ty + tz * tz);
+            const double sx = k2 * tx, sy = k2 * ty, sz = k2 * tz;
             const double px = mx + (my * tz - mz * ty), py = my + (mz * tx - mx * tz),
                          pz = mz + (mx * ty - my * tx);
             ux = mx + (py * sz - pz * sy) + h * E.x;
             uy = my + (pz * sx - px * sz) + h * E.y;
             uz = mz + (px * sy - py * sx) + h * E.z;
         }
-        double gam = sqrt(1.0 + ux * ux + uy * uy + uz * uz);
+        double g2 = 1.0 + ux * ux + uy * uy + uz * uz;
+        double ig = rsqrt64(g2);
+        const double gam = root_of(g2, ig);
         const double Ex = E.x, Ey = E.y, Ez = E.z, Bx = B.x, By = B.y, Bz = B.z;
         sink.tables();  // tables are needed from here on
-        const double chi = chi_e64(Ex, Ey, Ez, Bx, By, Bz, ux, uy, uz, gam, a.a_S);
+        const double chi = chi_e64(Ex, Ey, Ez, Bx, By, Bz, ux, uy, uz, gam, a.inv_aS);
         sink.chi(chi);
         double dvx = 0.0, dvy = 0.0, dvz = 0.0;
 
         if (chi < P.chi_th) {
             // ---- Sokolov continuous regime (Eq. 4, P_rad of Eq. 5)
             o.cont = true;
-            const double vx = ux / gam, vy = uy / gam, vz = uz / gam;
+            const double vx = ux * ig, vy = uy * ig, vz = uz * ig;
             const double fx = q * (Ex + (vy * Bz - vz * By));
             const double fy = q * (Ey + (vz * Bx - vx * Bz));
             const double fz = q * (Ez + (vx * By - vy * Bx));
             const double vf = vx * fx + vy * fy + vz * fz;
-            const double den = 1.0 + a.tau0w * vf;
-            dvx = a.tau0w * (fx - vx * vf) / den;
-            dvy = a.tau0w * (fy - vy * vf) / den;
-            dvz = a.tau0w * (fz - vz * vf) / den;
+            const double k = a.tau0w * rcp64(1.0 + a.tau0w * vf);
+            dvx = k * (fx - vx * vf);
+            dvy = k * (fy - vy * vf);
+            dvz = k * (fz - vz * vf);
             const double prad = a.C_rate * rate64<1>(G, chi, clamped);
             ux = ux + dt * (q * (dvy * Bz - dvz * By) - prad * vx);
             uy = uy + dt * (q * (dvz * Bx - dvx * Bz) - prad * vy);
             uz = uz + dt * (q * (dvx * By - dvy * Bx) - prad * vz);
-            gam = sqrt(1.0 + ux * ux + uy * uy + uz * uz);
+            ig = rsqrt64(1.0 + ux * ux + uy * uy + uz * uz);
         } else {
             // ---- optical depth (Eq. 6)
             const double Hv = rate64<0>(H, chi, clamped);
-            const double dtau = a.C_rate * Hv / gam * dt;
+            const double dtau = a.C_rate * Hv * ig * dt;
             if (dtau > 0.0 && !(tau > dtau)) {
                 o.clamped = clamped;
                 mid = {ux, uy, uz, gam, chi, dtau, E, B};
@@ -461,7 +463,7 @@ __device__ __forceinline__ bool lepton_push(const StepArgs &a, const Problem &P,
             tau = tau - dtau;
         }
         o.clamped = clamped;
-        mid = {ux, uy, uz, gam, tau, 0.0, {dvx, dvy, dvz}, {0.0, 0.0, 0.0}};
+        mid = {ux, uy, uz, ig, tau, 0.0, {dvx, dvy, dvz}, {0.0, 0.0, 0.0}};
     } else {
         // ---- mixed precision: FP32 physics; the FP64 state is read once,
         // increments are formed in FP32 and added back by integer
@@ -548,9 +550,9 @@ __device__ __forceinline__ void lepton_finish(const Problem &P, const LeptonStat
 {
     const Vec3<R> &dv = mid.E;
     if constexpr (PREC == kFP64) {
-        sink.template put<0>(s.x + P.dt * (mid.ux / mid.gam + dv.x));
-        sink.template put<1>(s.y + P.dt * (mid.uy / mid.gam + dv.y));
-        if (sink.has_z()) sink.template put<2>(s.z + P.dt * (mid.uz / mid.gam + dv.z));
+        sink.template put<0>(s.x + P.dt * (mid.ux * mid.gam + dv.x));
+        sink.template put<1>(s.y + P.dt * (mid.uy * mid.gam + dv.y));
+        if (sink.has_z()) sink.template put<2>(s.z + P.dt * (mid.uz * mid.gam + dv.z));
         sink.template put<3>(mid.ux);
         sink.template put<4>(mid.uy);
         sink.template put<5>(mid.uz);
@@ -583,18 +585,19 @@ __device__ __forceinline__ void lepton_events(const StepArgs &a, const Problem &
         const double dt = P.dt;
         double ux = mid.ux, uy = mid.uy, uz = mid.uz, gam = mid.gam, chi = mid.chi;
         double tau = s.tau, e_sub = 0.0;
-        double r = 1.0, wdt = mid.wdt;
+        double r = 1.0, wdt = mid.wdt, ig = 0.0;
         for (int k = 0;;) {
-            r = r - tau / wdt;
+            r = r - tau * rcp64(wdt);
             // ---- emission: Eq. 7 sampling, Eq. 8 recoil
             const uint4 rr = draw(P.seed, sp, kRngEmit, particle_id(S, i), tm.step, k);
             const double xi_p = u53(rr.x, rr.y), xi = u53(rr.z, rr.w);
-            const double ufrac = sample_cdf<double>(a.tab.Cg, a.tab.Gg, chi, xi_p, kSgMin, kSgSpan,
+            const double ufrac = sample_cdf(a.tab.Cg, a.tab.Gg, chi, xi_p, kSgMin, kSgSpan,
                                                     true, clamped);
-            const double pmag = sqrt(ux * ux + uy * uy + uz * uz);
+            const double p2 = ux * ux + uy * uy + uz * uz;
+            const double ip = p2 > 0.0 ? rsqrt64(p2) : 0.0, pmag = root_of(p2, ip);
             double gg = ufrac * gam;
             if (gg > pmag) gg = pmag;
-            if (n_emit == 0 && pmag > 0.0) sink.direction(ux / pmag, uy / pmag, uz / pmag);
+            if (n_emit == 0 && pmag > 0.0) sink.direction(ux * ip, uy * ip, uz * ip);
             ++n_emit;
             if (gg > P.gmin) {
                 sink.photon(nph, gg, k);
@@ -604,17 +607,19 @@ __device__ __forceinline__ void lepton_events(const StepArgs &a, const Problem &
                 e_sub += gg;
             }
             if (pmag > 0.0) {
-                const double scale = (pmag - gg) / pmag;
+                const double scale = (pmag - gg) * ip;
                 ux *= scale;
                 uy *= scale;
                 uz *= scale;
             }
             tau = -log(xi);
-            gam = sqrt(1.0 + ux * ux + uy * uy + uz * uz);
-            chi = chi_e64(E.x, E.y, E.z, B.x, B.y, B.z, ux, uy, uz, gam, a.a_S);
+            const double g2 = 1.0 + ux * ux + uy * uy + uz * uz;
+            ig = rsqrt64(g2);
+            gam = root_of(g2, ig);
+            chi = chi_e64(E.x, E.y, E.z, B.x, B.y, B.z, ux, uy, uz, gam, a.inv_aS);
             // ---- the rest of the step (Eq. 6)
             const double Hv = rate64<0>(H, chi, clamped);
-            wdt = a.C_rate * Hv / gam * dt;
+            wdt = a.C_rate * Hv * ig * dt;
             const double dtau = wdt * r;
             const bool more = dtau > 0.0 && !(tau > dtau);
             sat = more && ++k == P.max_emit;
@@ -625,9 +630,9 @@ __device__ __forceinline__ void lepton_events(const StepArgs &a, const Problem &
         }
         // ---- position (Eq. 4)
         if (nph) sink.origin(s.x, s.y, s.z);
-        sink.template put<0>(s.x + dt * (ux / gam));
-        sink.template put<1>(s.y + dt * (uy / gam));
-        if (sink.has_z()) sink.template put<2>(s.z + dt * (uz / gam));
+        sink.template put<0>(s.x + dt * (ux * ig));
+        sink.template put<1>(s.y + dt * (uy * ig));
+        if (sink.has_z()) sink.template put<2>(s.z + dt * (uz * ig));
         sink.template put<3>(ux);
         sink.template put<4>(uy);
         sink.template put<5>(uz);
@@ -986,13 +991,13 @@ __device__ __forceinline__ void write_photons(const Problem &P, const StepTime &
 // the fused steps), with every rounding explicit (a product left to the
 // compiler could be fused into the add in one place and hoisted out of a
 // loop in the other), so both give the same bits.
-__device__ __forceinline__ double photon_speed64(double ux, double uy, double uz)
+__device__ __forceinline__ double photon_u64(double ux, double uy, double uz)
 {
-    return __dsqrt_rn(__fma_rn(uz, uz, __fma_rn(uy, uy, __dmul_rn(ux, ux))));
+    return __fma_rn(uz, uz, __fma_rn(uy, uy, __dmul_rn(ux, ux)));  // |u|^2
 }
-__device__ __forceinline__ double photon_move64(double x, double u, double g, double dt)
+__device__ __forceinline__ double photon_move64(double x, double u, double ig, double dt)
 {
-    return __fma_rn(dt, __ddiv_rn(u, g), x);
+    return __fma_rn(dt, __dmul_rn(u, ig), x);  // ig = 1/|u|
 }
 __device__ __forceinline__ float photon_speed32(float fx, float fy, float fz)
 {
@@ -1022,20 +1027,23 @@ __device__ __forceinline__ bool photon_step(const StepArgs &a, const Problem &P,
     const double gux = Ph.ux[i], guy = Ph.uy[i], guz = Ph.uz[i];
     if (!(taud >= 0.0)) return false;
     if constexpr (PREC == kFP64) {
-        const double g = photon_speed64(gux, guy, guz);
+        const double u2 = photon_u64(gux, guy, guz);
+        const double ig = u2 > 0.0 ? rsqrt64(u2) : 0.0;
         const double dt = P.dt;
-        if (pairs && g > 2.0) {
+        if (pairs && u2 > 4.0) {
             Vec3<R> E, B;
-            eval_field<FK, R>(P.f, px, py, pz, tm.t, E, B);
-            const double kx = gux / g, ky = guy / g, kz = guz / g;
+            eval_field<FK>(P.f, px, py, pz, tm.t, E, B);
+            const double kx = gux * ig, ky = guy * ig, kz = guz * ig;
             const double ax = E.x + (ky * B.z - kz * B.y);
             const double ay = E.y + (kz * B.x - kx * B.z);
             const double az = E.z + (kx * B.y - ky * B.x);
             const double ke = kx * E.x + ky * E.y + kz * E.z;
             const double s = ax * ax + ay * ay + az * az - ke * ke;
-            const double chi = s > 0.0 ? g * sqrt(s) / a.a_S : 0.0;
+            // |u| sqrt(s) as one root
+            const double us = u2 * s;
+            const double chi = us > 0.0 ? root_of(us, rsqrt64(us)) * a.inv_aS : 0.0;
             const double Tr = rate64<2>(T, chi, clamped);
-            const double dtau = a.C_rate * Tr / g * dt;
+            const double dtau = a.C_rate * Tr * ig * dt;
             if (Ph.chi) Ph.chi[i] = chi;
             if (dtau > 0.0 && !(taud > dtau)) {
                 decayed = true;
@@ -1045,10 +1053,10 @@ __device__ __forceinline__ bool photon_step(const StepArgs &a, const Problem &P,
                 Ph.tau[i] = taud - dtau;
             }
         }
-        if (!decayed && g > 0.0) {
-            Ph.x[i] = photon_move64(px, gux, g, dt);
-            Ph.y[i] = photon_move64(py, guy, g, dt);
-            if (Ph.z) Ph.z[i] = photon_move64(pz, guz, g, dt);
+        if (!decayed && u2 > 0.0) {
+            Ph.x[i] = photon_move64(px, gux, ig, dt);
+            Ph.y[i] = photon_move64(py, guy, ig, dt);
+            if (Ph.z) Ph.z[i] = photon_move64(pz, guz, ig, dt);
         }
     } else {
         // ---- mixed precision: FP32 physics, FP64 accumulation by
@@ -1120,7 +1128,7 @@ __device__ __forceinline__ void write_pairs(const StepArgs &a, const Problem &P,
             double v, om, tm, tp;
             bool clamped = false;  // counted with the rate, at the same chi
             if constexpr (PREC == kFP64) {
-                v = sample_cdf<double>(a.tab.Cp, a.tab.Gp, chi, u53(r1.x, r1.y), kSpMin, kSpSpan,
+                v = sample_cdf(a.tab.Cp, a.tab.Gp, chi, u53(r1.x, r1.y), kSpMin, kSpSpan,
                                        false, clamped);
                 om = 1.0 - v;
                 tm = -log(u53(r1.z, r1.w));
@@ -2444,13 +2452,15 @@ __global__ void __launch_bounds__(256) k_fused_photons(const __grid_constant__ F
         }
         if (moves > 0 && tau >= 0.0) {
             if constexpr (PREC == kFP64) {
-                const double g = photon_speed64(ux, uy, uz);
-                if (g > 0.0)
+                const double u2 = photon_u64(ux, uy, uz);
+                if (u2 > 0.0) {
+                    const double ig = rsqrt64(u2);
                     for (int m = 0; m < moves; ++m) {
-                        x = photon_move64(x, ux, g, P.dt);
-                        y = photon_move64(y, uy, g, P.dt);
-                        z = photon_move64(z, uz, g, P.dt);
+                        x = photon_move64(x, ux, ig, P.dt);
+                        y = photon_move64(y, uy, ig, P.dt);
+                        z = photon_move64(z, uz, ig, P.dt);
                     }
+                }
             } else {
                 const float fx = hi_d(ux), fy = hi_d(uy), fz = hi_d(uz);
                 const float g = photon_speed32(fx, fy, fz);
