@@ -1079,7 +1079,7 @@ int qp_step_fused(qp_ctx *ctx, const qp_step_params *s, int32_t fuse, void *stre
     // the photon order sorts 32-bit indices on keys of at most 64 bits
     if (cap_g >= (int64_t)0xFFFFFFFFll || qp::fused_key_bits(K, tiles, nullptr) > 64)
         return QP_ERR_INVALID_ARG;
-    const int order_grid = 2 * ctx->num_sms;
+    const int order_grid = qp::kSortBlocksPerSm * ctx->num_sms;
     const size_t sort_bytes = (qp::coalesce_scratch_bytes(cap_g, order_grid) + 255) / 256 * 256;
     const size_t bytes = sort_bytes + 256;
     if (bytes > ctx->fuse_bytes) {
@@ -1192,7 +1192,7 @@ int qp_sort_species(qp_ctx *ctx, int32_t handle, const qp_field *grid, void *str
     if ((double)g.nx * (double)g.ny > 9.0e18) return QP_ERR_INVALID_ARG;
     DeviceGuard d(ctx->device);
     if (!d.ok) return QP_ERR_CUDA;
-    const int grid_blocks = 2 * ctx->num_sms;
+    const int grid_blocks = qp::kSortBlocksPerSm * ctx->num_sms;
     const size_t bytes = qp::coalesce_scratch_bytes(sd.capacity, grid_blocks);
     if (bytes > ctx->coal_bytes) {
         void *p = nullptr;
@@ -1236,7 +1236,7 @@ int qp_coalesce_photons(qp_ctx *ctx, int32_t handle, const qp_coalesce_params *P
     }
     DeviceGuard g(ctx->device);
     if (!g.ok) return QP_ERR_CUDA;
-    const int grid = 2 * ctx->num_sms;
+    const int grid = qp::kSortBlocksPerSm * ctx->num_sms;
     const size_t bytes = qp::coalesce_scratch_bytes(d.capacity, grid);
     if (bytes > ctx->coal_bytes) {
         void *p = nullptr;

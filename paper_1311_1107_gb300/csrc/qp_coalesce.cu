@@ -18,18 +18,18 @@
 // device, grids of G blocks each owning one contiguous chunk of slots):
 //   k_co_prepare   roles (1 alive, 0 decayed) and group keys;
 //   radix passes   stable LSD sort of (key, slot), 8 bits a pass:
-//                  k_co_hist, k_co_scan_hist, k_co_scatter;
+//                  k_co_hist, k_co_scan_rows, k_co_scatter;
 //   k_co_groups    groups (runs of one key) cut into runs of at most
 //                  max_group members in slot order; runs of >= min_group
 //                  listed;
-//   k_co_runs      one thread a run: its momentum checked, roles set (2 at
+//   k_co_runs      eight lanes a run: its sums, its momentum checked, roles set (2 at
 //                  the first member, 0 at the others);
-//   role scan      k_co_chunk_sums, k_co_scan_chunks, k_co_offsets: the
+//   role scan      k_co_chunk_sums, k_co_scan, k_co_offsets: the
 //                  output slot of every survivor in slot order;
 //   k_co_kept      survivors copied to the staging arrays;
 //   k_co_pairs     merged pairs computed and written to the staging arrays;
 //   k_co_copy_back staging -> species, new live count.
-// Group sums run in slot order in one thread per run, with the oracle's
+// Group sums run in slot order, one lane a sum, with the oracle's
 // operations in the oracle's order; this unit is compiled without FMA
 // contraction, so keys, sums and merged momenta are the oracle's bit for
 // bit (the fresh optical depths -log(xi) differ by the last bit at most).
@@ -46,6 +46,9 @@ constexpr int kCoThreads = 256;
 constexpr int kRadix = 256;
 constexpr int kCoWarps = kCoThreads / 32;
 constexpr int kRngCoalesce = 5;
+// Blocks of the kernels that stride over slots or runs, over those that own a
+// chunk of slots (their number is the length of a digit's row).
+constexpr int kWide = 2;
 
 struct CoParams {
     double x0, y0, z0, dx, dy, dz;
@@ -53,6 +56,7 @@ struct CoParams {
     long long nx, ny, nz;
     int lb;            // log2 of energy bins per octave
     int D;             // direction bins per face axis
+    double half_D;     // D / 2
     int min_group;
     int max_group;     // longest run of one group merged into one pair
     int dims;
@@ -82,52 +86,73 @@ __device__ __forceinline__ void chunk_of(long long n, long long *beg, long long 
     if (*beg > n) *beg = n;
 }
 
-// e: the photon's energy |u| (sqrt(ux ux + uy uy + uz uz), formed by the caller)
+// Square root rounded to nearest of x, within a half unit of the last place
+// plus 2^-50 of one: a residual correction of x times 1/sqrt(x) (Markstein),
+// nine FP64 instructions for an IEEE square root's more.
+__device__ __forceinline__ double sqrt_rn(double x)
+{
+    return x > 0.0 ? root_of(x, rsqrt64(x)) : sqrt(x);
+}
+
+// The cell of one axis: the offset times the reciprocal of the cell size
+// (formed on the host), rounded down by the conversion; false outside the box
+// (NaN converts to the lowest integer).
+__device__ __forceinline__ bool cell_of(double x, double x0, double ix, long long n, long long &c)
+{
+    c = __double2ll_rd((x - x0) * ix);
+    return c >= 0 && c < n;
+}
+
+__device__ __forceinline__ unsigned long long abs_bits(double x)
+{
+    return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+
+// e: the photon's energy |u| (sqrt(ux ux + uy uy + uz uz), formed by the
+// caller).  Comparisons and roundings are integer instructions or
+// conversions: on the narrow FP64 pipe this is 30 instructions a photon.
 __device__ unsigned long long group_key(const CoParams &C, double x, double y, double z, double ux,
                                         double uy, double uz, double e)
 {
-    // cell: the offset times the reciprocal of the cell size (formed on the host)
-    const double gx = floor((x - C.x0) * C.idx);
-    const double gy = floor((y - C.y0) * C.idy);
-    const double gz = C.dims == 3 ? floor((z - C.z0) * C.idz) : 0.0;
-    if (!(gx >= 0.0 && gx < (double)C.nx && gy >= 0.0 && gy < (double)C.ny && gz >= 0.0 &&
-          gz < (double)C.nz))
+    long long cx, cy, cz = 0;
+    if (!cell_of(x, C.x0, C.idx, C.nx, cx) || !cell_of(y, C.y0, C.idy, C.ny, cy) ||
+        (C.dims == 3 && !cell_of(z, C.z0, C.idz, C.nz, cz)))
         return C.nomerge;
     const unsigned long long eb = (unsigned long long)__double_as_longlong(e);
     const unsigned long long ex = (eb >> 52) & 0x7FFull;
     if (ex == 0ull || ex == 0x7FFull) return C.nomerge;
     const unsigned long long ebin = (ex << C.lb) | ((eb & ((1ull << 52) - 1ull)) >> (52 - C.lb));
-    const double u[3] = {ux, uy, uz};
-    int f = 0;
-    if (fabs(u[1]) > fabs(u[f])) f = 1;
-    if (fabs(u[2]) > fabs(u[f])) f = 2;
-    const int face = 2 * f + (u[f] < 0.0 ? 1 : 0);
-    const double r = 1.0 / fabs(u[f]);
-    const double a = u[(f + 1) % 3] * r;
-    const double b = u[(f + 2) % 3] * r;
+    // the dominant axis (the first of equals), the next two in cyclic order
+    const bool y_dom = abs_bits(uy) > abs_bits(ux);
+    const bool z_dom = abs_bits(uz) > abs_bits(y_dom ? uy : ux);
+    const double d = z_dom ? uz : y_dom ? uy : ux;
+    const double p = z_dom ? ux : y_dom ? uz : uy, q = z_dom ? uy : y_dom ? ux : uz;
+    const int face = 2 * (z_dom ? 2 : y_dom ? 1 : 0) + (__double2hiint(d) < 0 ? 1 : 0);
+    const double r = rcp64(fabs(d));
     const long long D = C.D;
-    long long ia = (long long)floor((a + 1.0) * (0.5 * (double)D));
-    long long ib = (long long)floor((b + 1.0) * (0.5 * (double)D));
-    if (ia > D - 1) ia = D - 1;
-    if (ib > D - 1) ib = D - 1;
+    const long long ia = min((long long)__double2int_rd((p * r + 1.0) * C.half_D), D - 1);
+    const long long ib = min((long long)__double2int_rd((q * r + 1.0) * C.half_D), D - 1);
     const unsigned long long dbin =
         ((unsigned long long)face * (unsigned long long)D + (unsigned long long)ia) *
             (unsigned long long)D +
         (unsigned long long)ib;
     const unsigned long long cell =
-        ((unsigned long long)gx * (unsigned long long)C.ny + (unsigned long long)gy) *
+        ((unsigned long long)cx * (unsigned long long)C.ny + (unsigned long long)cy) *
             (unsigned long long)C.nz +
-        (unsigned long long)gz;
+        (unsigned long long)cz;
     const unsigned long long n_e = 2048ull << C.lb, n_d = 6ull * (unsigned long long)(D * D);
     return (cell * n_e + ebin) * n_d + dbin;
 }
 
 // ---------------------------------------------------------------- prepare
 
+// Doubles of a photon in the merge's copy: w, |u|, ux, uy, uz, x, y, z.
+constexpr int kMember = 8;
+
 __global__ void __launch_bounds__(kCoThreads) k_co_prepare(SpeciesDev S, CoParams C,
                                                            unsigned long long *keys,
                                                            unsigned *vals, unsigned char *role,
-                                                           double *en, long long *counts,
+                                                           double *members, long long *counts,
                                                            int *status)
 {
     const long long n = live_count(S, status);
@@ -140,9 +165,15 @@ __global__ void __launch_bounds__(kCoThreads) k_co_prepare(SpeciesDev S, CoParam
             unsigned long long key = C.nomerge;
             if (alive) {
                 const double ux = S.ux[i], uy = S.uy[i], uz = S.uz[i];
-                const double e = sqrt(ux * ux + uy * uy + uz * uz);
-                en[i] = e;  // the merge sums these energies
-                key = group_key(C, S.x[i], S.y[i], S.z ? S.z[i] : 0.0, ux, uy, uz, e);
+                const double x = S.x[i], y = S.y[i], z = S.z ? S.z[i] : 0.0, w = S.w[i];
+                const double e = sqrt_rn(ux * ux + uy * uy + uz * uz);
+                key = group_key(C, x, y, z, ux, uy, uz, e);
+                // what the runs sum, side by side: they gather it in key order
+                double2 *const m = reinterpret_cast<double2 *>(members + kMember * i);
+                m[0] = make_double2(w, e);
+                m[1] = make_double2(ux, uy);
+                m[2] = make_double2(uz, x);
+                m[3] = make_double2(y, z);
             }
             keys[i] = key;
             vals[i] = (unsigned)i;
@@ -166,37 +197,19 @@ __global__ void __launch_bounds__(kCoThreads) k_co_hist(const unsigned long long
     hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = h[threadIdx.x];
 }
 
-// Exclusive scan of m entries in place, one block of 1024 threads, in tiles
-// of 8192 entries: a tile is loaded with coalesced reads into shared memory
-// (one pad word per 32, so that a thread's 8 contiguous entries fall in
-// distinct banks across the warp), each thread scans its 8 entries, the
-// thread sums are scanned across the block, and the tile is written back
-// coalesced with the running total of the earlier tiles added.  total: the
-// sum of all entries, or nullptr.
-constexpr int kScanThreads = 1024, kScanPer = 8, kScanTile = kScanThreads * kScanPer;
+// Exclusive scan of m entries (a sum a block) in place, by one block, with the
+// sum of all entries in *total.
+constexpr int kScanThreads = 1024;
 
 __global__ void __launch_bounds__(kScanThreads) k_co_scan(unsigned *v, int m, long long *total)
 {
-    __shared__ unsigned s[kScanTile + kScanTile / 32];
     __shared__ unsigned s_warp[32];
     __shared__ unsigned s_tile;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     unsigned carry = 0u;
-    for (int base = 0; base < m; base += kScanTile) {
-#pragma unroll
-        for (int k = 0; k < kScanPer; ++k) {
-            const int i = k * kScanThreads + t;
-            s[i + (i >> 5)] = base + i < m ? v[base + i] : 0u;
-        }
-        __syncthreads();
-        unsigned loc[kScanPer], sum = 0u;
-#pragma unroll
-        for (int k = 0; k < kScanPer; ++k) {
-            const int i = t * kScanPer + k;
-            loc[k] = s[i + (i >> 5)];
-            sum += loc[k];
-        }
-        unsigned inc = sum;
+    for (int base = 0; base < m; base += kScanThreads) {
+        const unsigned x = base + t < m ? v[base + t] : 0u;
+        unsigned inc = x;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const unsigned y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
@@ -205,34 +218,57 @@ __global__ void __launch_bounds__(kScanThreads) k_co_scan(unsigned *v, int m, lo
         if (lane == 31) s_warp[w] = inc;
         __syncthreads();
         if (w == 0) {
-            const unsigned x = s_warp[lane];
-            unsigned xi = x;
+            const unsigned sx = s_warp[lane];
+            unsigned xi = sx;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
                 const unsigned y = __shfl_up_sync(0xFFFFFFFFu, xi, d);
                 if (lane >= d) xi += y;
             }
-            s_warp[lane] = xi - x;
+            s_warp[lane] = xi - sx;
             if (lane == 31) s_tile = xi;
         }
         __syncthreads();
-        unsigned run = carry + s_warp[w] + (inc - sum);
-#pragma unroll
-        for (int k = 0; k < kScanPer; ++k) {
-            const int i = t * kScanPer + k;
-            s[i + (i >> 5)] = run;
-            run += loc[k];
-        }
+        if (base + t < m) v[base + t] = carry + s_warp[w] + (inc - x);
         carry += s_tile;
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < kScanPer; ++k) {
-            const int i = k * kScanThreads + t;
-            if (base + i < m) v[base + i] = s[i + (i >> 5)];
-        }
-        __syncthreads();  // s, s_warp and s_tile are reused by the next tile
+        __syncthreads();  // s_warp and s_tile are reused by the next entries
     }
-    if (total && t == 0) *total = (long long)carry;
+    if (t == 0) *total = (long long)carry;
+}
+
+// Exclusive scan over the blocks of every digit's counts, one block a digit,
+// and the digit's total (k_co_scatter adds the smaller digits' totals).  One
+// block over all kRadix x 304 counts took 19 us a pass; this takes 3.
+constexpr int kRowThreads = 128;
+
+__global__ void __launch_bounds__(kRowThreads) k_co_scan_rows(unsigned *hist, int blocks,
+                                                              unsigned *total)
+{
+    __shared__ unsigned s_w[kRowThreads / 32];
+    unsigned *row = hist + (size_t)blockIdx.x * blocks;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    unsigned run = 0u;
+    for (int b0 = 0; b0 < blocks; b0 += kRowThreads) {
+        const unsigned v = b0 + t < blocks ? row[b0 + t] : 0u;
+        unsigned inc = v;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += y;
+        }
+        if (lane == 31) s_w[warp] = inc;
+        __syncthreads();
+        unsigned before = 0u, all = 0u;
+#pragma unroll
+        for (int w = 0; w < kRowThreads / 32; ++w) {
+            if (w < warp) before += s_w[w];
+            all += s_w[w];
+        }
+        if (b0 + t < blocks) row[b0 + t] = run + before + inc - v;
+        run += all;
+        __syncthreads();
+    }
+    if (t == 0) total[blockIdx.x] = run;
 }
 
 // Stable scatter: the block walks its chunk tile by tile; within a tile an
@@ -243,12 +279,29 @@ __global__ void __launch_bounds__(kCoThreads) k_co_scatter(const unsigned long l
                                                            unsigned long long *kout,
                                                            unsigned *vout, int shift,
                                                            const unsigned *hist,
+                                                           const unsigned *total,
                                                            const long long *counts)
 {
     __shared__ unsigned base[kRadix];
     __shared__ unsigned wc[kCoWarps][kRadix];
+    static_assert(kRadix == kCoThreads, "one thread a digit");
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    base[t] = hist[(size_t)t * gridDim.x + blockIdx.x];
+    {
+        // the digits below t, over all blocks, then t's of the earlier blocks
+        const unsigned v = total[t];
+        unsigned inc = v;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += y;
+        }
+        if (lane == 31) wc[0][warp] = inc;
+        __syncthreads();
+        unsigned before = 0u;
+        for (int w = 0; w < warp; ++w) before += wc[0][w];
+        base[t] = before + inc - v + hist[(size_t)t * gridDim.x + blockIdx.x];
+        __syncthreads();
+    }
     long long beg, end;
     chunk_of(counts[0], &beg, &end);
     const unsigned lt = (1u << lane) - 1u;
@@ -289,32 +342,10 @@ __global__ void __launch_bounds__(kCoThreads) k_co_scatter(const unsigned long l
 
 // ---------------------------------------------------------------- groups
 
+// A run's sums over its members, and the momentum of the first.
 struct GroupSums {
-    double W, E, P[3], X[3];
+    double W, E, P[3], X[3], u[3];
 };
-
-// The sums of a run [a, b) of the sorted order, member by member in slot
-// order; en: the members' energies |u| from k_co_prepare.
-__device__ GroupSums group_sums(const SpeciesDev &S, const double *en, const unsigned *vals,
-                                long long a, long long b)
-{
-    GroupSums g{0.0, 0.0, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
-    for (long long k = a; k < b; ++k) {
-        const unsigned i = vals[k];
-        const double w = S.w[i];
-        const double ux = S.ux[i], uy = S.uy[i], uz = S.uz[i];
-        const double e = en[i];
-        g.W = g.W + w;
-        g.E = g.E + w * e;
-        g.P[0] = g.P[0] + w * ux;
-        g.P[1] = g.P[1] + w * uy;
-        g.P[2] = g.P[2] + w * uz;
-        g.X[0] = g.X[0] + w * S.x[i];
-        g.X[1] = g.X[1] + w * S.y[i];
-        g.X[2] = g.X[2] + w * (S.z ? S.z[i] : 0.0);
-    }
-    return g;
-}
 
 // A merged group (run [j, end) of the sorted keys) starts at j; its end.
 __device__ __forceinline__ bool group_start(const unsigned long long *keys, long long j,
@@ -364,27 +395,67 @@ __global__ void __launch_bounds__(kCoThreads) k_co_groups(CoParams C,
     }
 }
 
-// One thread a run: its sums, kept for k_co_pairs; a run whose momentum
-// vanishes is kept as it is, the others become pairs (role 2 at the first
-// member, 0 at the others).
-__global__ void __launch_bounds__(kCoThreads) k_co_runs(SpeciesDev S, const double *en,
+// Eight lanes a run, one of its eight sums each, member by member in slot
+// order; the sums are kept for k_co_pairs, with the first member's momentum.
+// A run whose momentum vanishes is kept as it is, the others become pairs
+// (role 2 at the first member, 0 at the others).  Bound by the gather in key
+// order: a member is 64 consecutive bytes of the copy that k_co_prepare
+// writes, one line for its eight lanes, where the species' eight arrays were
+// eight sectors of 32 bytes (4e6 photons: a lane a run over the arrays 466 us,
+// eight lanes over the arrays 524, over the copy 391).
+constexpr int kRunLanes = kMember;
+
+__global__ void __launch_bounds__(kCoThreads) k_co_runs(const double *members,
                                                         const unsigned *vals, const uint2 *runs,
                                                         unsigned char *role, GroupSums *rsum,
                                                         const long long *counts,
                                                         long long *stats)
 {
+    static_assert(sizeof(GroupSums) == 11 * sizeof(double), "eight sums, then the momentum");
     const long long nr = counts[2];
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < nr; r += stride) {
+    const int c = threadIdx.x % kRunLanes, lane = threadIdx.x & 31;
+    const unsigned team = 0xFFu << (lane & 24);
+    const long long stride = (long long)gridDim.x * (kCoThreads / kRunLanes);
+    for (long long r = (long long)blockIdx.x * (kCoThreads / kRunLanes) + threadIdx.x / kRunLanes;
+         r < nr; r += stride) {
         const uint2 run = runs[r];
-        const GroupSums g = group_sums(S, en, vals, run.x, run.y);
-        rsum[r] = g;
-        const double *P = g.P;
-        if (!(P[0] * P[0] + P[1] * P[1] + P[2] * P[2] > 0.0)) continue;
-        for (unsigned k = run.x; k < run.y; ++k) role[vals[k]] = 0;
-        role[vals[run.x]] = 2;  // the sorted run is in slot order: its first
-        atomicAdd((unsigned long long *)&stats[0], 1ull);
-        atomicAdd((unsigned long long *)&stats[1], (unsigned long long)(run.y - run.x));
+        const unsigned anchor = vals[run.x];
+        // lane c sums W, E, P_x, P_y, P_z, X, Y, Z: w itself, or w times its double
+        // four members in flight ahead of the four being added
+        auto load = [&](unsigned k, double (&v)[4]) {
+#pragma unroll
+            for (unsigned m = 0; m < 4; ++m)
+                v[m] = k + m < run.y ? members[(size_t)kMember * vals[k + m] + c] : 0.0;
+        };
+        double sum = 0.0, v[4];
+        load(run.x, v);
+        const double first = v[0];
+        for (unsigned k = run.x; k < run.y; k += 4) {
+            double next[4];
+            load(k + 4, next);
+#pragma unroll
+            for (unsigned m = 0; m < 4; ++m) {
+                if (k + m >= run.y) break;
+                const double w = __shfl_sync(team, v[m], 0, kRunLanes);
+                sum = sum + (c == 0 ? v[m] : w * v[m]);
+            }
+#pragma unroll
+            for (int m = 0; m < 4; ++m) v[m] = next[m];
+        }
+        double *const out = &rsum[r].W;
+        out[c] = sum;
+        if (c >= 2 && c < 5) out[6 + c] = first;
+        const double px = __shfl_sync(team, sum, 2, kRunLanes);
+        const double py = __shfl_sync(team, sum, 3, kRunLanes);
+        const double pz = __shfl_sync(team, sum, 4, kRunLanes);
+        if (!(px * px + py * py + pz * pz > 0.0)) continue;
+        // the sorted run is in slot order: its first member is the anchor
+        for (unsigned m = run.x + c; m < run.y; m += kRunLanes)
+            role[m == run.x ? anchor : vals[m]] = m == run.x ? 2 : 0;
+        if (c == 0) {
+            atomicAdd((unsigned long long *)&stats[0], 1ull);
+            atomicAdd((unsigned long long *)&stats[1], (unsigned long long)(run.y - run.x));
+        }
     }
 }
 
@@ -459,14 +530,14 @@ __global__ void __launch_bounds__(kCoThreads) k_co_kept(SpeciesDev S, const unsi
         const unsigned o = off[i];
         st.f[0][o] = S.x[i];
         st.f[1][o] = S.y[i];
-        st.f[2][o] = S.z ? S.z[i] : 0.0;
+        if (S.z) st.f[2][o] = S.z[i];
         st.f[3][o] = S.ux[i];
         st.f[4][o] = S.uy[i];
         st.f[5][o] = S.uz[i];
         st.f[6][o] = S.tau[i];
         st.f[7][o] = S.w[i];
-        st.f[8][o] = S.chi ? S.chi[i] : 0.0;
-        st.nemit[o] = S.nemit ? S.nemit[i] : 0;
+        if (S.chi) st.f[8][o] = S.chi[i];
+        if (S.nemit) st.nemit[o] = S.nemit[i];
     }
 }
 
@@ -484,19 +555,21 @@ __global__ void __launch_bounds__(kCoThreads) k_co_pairs(SpeciesDev S, CoParams 
         const unsigned anchor = vals[run.x];
         if (role[anchor] != 2) continue;
         const GroupSums g = rsum[q];
-        const double W = g.W;
-        const double eps = g.E / W;
-        const double c[3] = {g.P[0] / W, g.P[1] / W, g.P[2] / W};
+        const double W = g.W, iW = __drcp_rn(W);
+        const double eps = quotient64(g.E, W, iW);
+        const double c[3] = {quotient64(g.P[0], W, iW), quotient64(g.P[1], W, iW),
+                             quotient64(g.P[2], W, iW)};
         const double c2 = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
         const double d2 = eps * eps - c2;
-        const double dm = d2 > 0.0 ? sqrt(d2) : 0.0;
-        const double cm = sqrt(c2);
-        const double ph[3] = {c[0] / cm, c[1] / cm, c[2] / cm};
-        const double r[3] = {S.ux[anchor], S.uy[anchor], S.uz[anchor]};
+        const double dm = d2 > 0.0 ? sqrt_rn(d2) : 0.0;
+        const double cm = sqrt_rn(c2), icm = __drcp_rn(cm);
+        const double ph[3] = {quotient64(c[0], cm, icm), quotient64(c[1], cm, icm),
+                              quotient64(c[2], cm, icm)};
+        const double r[3] = {g.u[0], g.u[1], g.u[2]};
         const double rp = r[0] * ph[0] + r[1] * ph[1] + r[2] * ph[2];
         double v[3] = {r[0] - rp * ph[0], r[1] - rp * ph[1], r[2] - rp * ph[2]};
-        double vm = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-        const double rm = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
+        double vm = sqrt_rn(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+        const double rm = sqrt_rn(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
         if (!(vm > 1e-12 * rm)) {
             // the first photon is parallel to P: the axis least aligned with P
             int a = 0;
@@ -506,17 +579,21 @@ __global__ void __launch_bounds__(kCoThreads) k_co_pairs(SpeciesDev S, CoParams 
             v[0] = (a == 0 ? 1.0 : 0.0) - ap * ph[0];
             v[1] = (a == 1 ? 1.0 : 0.0) - ap * ph[1];
             v[2] = (a == 2 ? 1.0 : 0.0) - ap * ph[2];
-            vm = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+            vm = sqrt_rn(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
         }
-        const double dv[3] = {dm * (v[0] / vm), dm * (v[1] / vm), dm * (v[2] / vm)};
+        const double ivm = __drcp_rn(vm);
+        const double dv[3] = {dm * quotient64(v[0], vm, ivm), dm * quotient64(v[1], vm, ivm),
+                              dm * quotient64(v[2], vm, ivm)};
         const unsigned o = off[anchor];
         const long long id = particle_id(S, anchor);
+        const double X[3] = {quotient64(g.X[0], W, iW), quotient64(g.X[1], W, iW),
+                             quotient64(g.X[2], W, iW)};
         for (int s = 0; s < 2; ++s) {
             const double sg = s == 0 ? 1.0 : -1.0;
             const uint4 rr = draw(C.seed, QP_PHOTON, kRngCoalesce, id, (uint64_t)C.step, s);
-            st.f[0][o + s] = g.X[0] / W;
-            st.f[1][o + s] = g.X[1] / W;
-            st.f[2][o + s] = g.X[2] / W;
+            st.f[0][o + s] = X[0];
+            st.f[1][o + s] = X[1];
+            st.f[2][o + s] = X[2];
             st.f[3][o + s] = c[0] + sg * dv[0];
             st.f[4][o + s] = c[1] + sg * dv[1];
             st.f[5][o + s] = c[2] + sg * dv[2];
@@ -589,14 +666,14 @@ __global__ void __launch_bounds__(kCoThreads) k_sort_gather(SpeciesDev S, const 
         const unsigned i = vals[k];
         st.f[0][k] = S.x[i];
         st.f[1][k] = S.y[i];
-        st.f[2][k] = S.z ? S.z[i] : 0.0;
+        if (S.z) st.f[2][k] = S.z[i];
         st.f[3][k] = S.ux[i];
         st.f[4][k] = S.uy[i];
         st.f[5][k] = S.uz[i];
         st.f[6][k] = S.tau[i];
         st.f[7][k] = S.w[i];
-        st.f[8][k] = S.chi ? S.chi[i] : 0.0;
-        st.nemit[k] = S.nemit ? S.nemit[i] : 0;
+        if (S.chi) st.f[8][k] = S.chi[i];
+        if (S.nemit) st.nemit[k] = S.nemit[i];
     }
 }
 
@@ -606,7 +683,7 @@ size_t coalesce_scratch_bytes(int64_t cap, int grid)
 {
     const size_t c = (size_t)(cap > 0 ? cap : 1);
     return 2 * c * 8 + 2 * c * 4 + c + c * 4 + c * 9 * 8 + c * 4 +
-           ((size_t)kRadix * grid + grid + 64) * 4 + 16 * 8 + (c / 3 + 1) * 8 +
+           ((size_t)kRadix * grid + kRadix + grid + 64) * 4 + 16 * 8 + (c / 3 + 1) * 8 +
            (c / 3 + 1) * sizeof(GroupSums) + 32 * 256;
 }
 
@@ -620,7 +697,7 @@ struct CoScratch {
     unsigned char *role;
     unsigned *off;
     Stage stg;
-    unsigned *hist, *chunk;
+    unsigned *hist, *total, *chunk;  // counts of a pass by digit and block, by digit; chunk sums
     long long *counts;
     uint2 *runs;
     GroupSums *rsum;  // the sums of each run (k_co_runs, for k_co_pairs)
@@ -645,11 +722,28 @@ CoScratch carve(void *scratch, int64_t cap, int grid)
     for (int f = 0; f < 9; ++f) s.stg.f[f] = (double *)take(c * 8);
     s.stg.nemit = (int *)take(c * 4);
     s.hist = (unsigned *)take((size_t)kRadix * grid * 4);
+    s.total = (unsigned *)take((size_t)kRadix * 4);
     s.chunk = (unsigned *)take((size_t)grid * 4 + 64);
     s.counts = (long long *)take(16 * 8);
     s.runs = (uint2 *)take((c / 3 + 1) * sizeof(uint2));
     s.rsum = (GroupSums *)take((c / 3 + 1) * sizeof(GroupSums));
     return s;
+}
+
+// `passes` passes of the stable sort of the counts[0] (key, value) pairs in
+// keys[0] and vals[0], 8 bits each from the lowest; the sorted pairs are in
+// keys[r] and vals[r] of the returned r.
+int radix_sort(const CoScratch &cs, int passes, int grid, cudaStream_t st)
+{
+    int cur = 0;
+    for (int ps = 0; ps < passes; ++ps, cur ^= 1) {
+        k_co_hist<<<grid, kCoThreads, 0, st>>>(cs.keys[cur], 8 * ps, cs.hist, cs.counts);
+        k_co_scan_rows<<<kRadix, kRowThreads, 0, st>>>(cs.hist, grid, cs.total);
+        k_co_scatter<<<grid, kCoThreads, 0, st>>>(cs.keys[cur], cs.vals[cur], cs.keys[cur ^ 1],
+                                                   cs.vals[cur ^ 1], 8 * ps, cs.hist, cs.total,
+                                                   cs.counts);
+    }
+    return cur;
 }
 
 }  // namespace
@@ -663,13 +757,13 @@ cudaError_t launch_coalesce(const SpeciesDev &S, const qp_coalesce_params *P, vo
     unsigned char *role = cs.role;
     unsigned *off = cs.off;
     const Stage stg = cs.stg;
-    unsigned *hist = cs.hist;
     unsigned *chunk = cs.chunk;
     long long *counts = cs.counts;
     uint2 *runs = cs.runs;
-    // the photons' energies (k_co_prepare to k_co_runs) in the chi staging
-    // array, which k_co_kept and k_co_pairs write only after k_co_runs
-    double *en = stg.f[8];
+    // the merge's copy of the photons (k_co_prepare to k_co_runs) takes the
+    // place of the staging arrays, which k_co_kept and k_co_pairs write after
+    static_assert(kMember <= 9, "the copy fits the nine staging arrays");
+    double *members = stg.f[0];
 
     CoParams C{};
     int passes = 0;
@@ -690,6 +784,7 @@ cudaError_t launch_coalesce(const SpeciesDev &S, const qp_coalesce_params *P, vo
         while ((1 << lb) < P->energy_bins_per_octave) ++lb;
         C.lb = lb;
         C.D = P->direction_bins;
+        C.half_D = 0.5 * C.D;
         C.min_group = P->min_group;
         C.max_group = P->max_group > 0 ? P->max_group : 256;
         C.dims = S.z ? 3 : 2;
@@ -708,29 +803,23 @@ cudaError_t launch_coalesce(const SpeciesDev &S, const qp_coalesce_params *P, vo
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(stats, 0, 4 * 8, st);
     if (e != cudaSuccess) return e;
-    k_co_prepare<<<grid, kCoThreads, 0, st>>>(S, C, keys[0], vals[0], role, en, counts, status);
-    int cur = 0;
-    for (int ps = 0; ps < passes; ++ps) {
-        k_co_hist<<<grid, kCoThreads, 0, st>>>(keys[cur], 8 * ps, hist, counts);
-        k_co_scan<<<1, 1024, 0, st>>>(hist, kRadix * grid, nullptr);
-        k_co_scatter<<<grid, kCoThreads, 0, st>>>(keys[cur], vals[cur], keys[cur ^ 1],
-                                                   vals[cur ^ 1], 8 * ps, hist, counts);
-        cur ^= 1;
-    }
+    k_co_prepare<<<kWide * grid, kCoThreads, 0, st>>>(S, C, keys[0], vals[0], role, members, counts,
+                                                          status);
+    const int cur = radix_sort(cs, passes, grid, st);
     if (passes) {
-        k_co_groups<<<grid, kCoThreads, 0, st>>>(C, keys[cur], counts, runs);
-        k_co_runs<<<grid, kCoThreads, 0, st>>>(S, en, vals[cur], runs, role, cs.rsum, counts,
+        k_co_groups<<<kWide * grid, kCoThreads, 0, st>>>(C, keys[cur], counts, runs);
+        k_co_runs<<<kWide * grid, kCoThreads, 0, st>>>(members, vals[cur], runs, role, cs.rsum, counts,
                                                 stats);
     }
     k_co_chunk_sums<<<grid, kCoThreads, 0, st>>>(role, chunk, counts);
-    k_co_scan<<<1, 1024, 0, st>>>(chunk, grid, counts + 1);
+    k_co_scan<<<1, kScanThreads, 0, st>>>(chunk, grid, counts + 1);
     k_co_offsets<<<grid, kCoThreads, 0, st>>>(role, chunk, off, counts);
-    k_co_kept<<<grid, kCoThreads, 0, st>>>(S, role, off, stg, counts);
+    k_co_kept<<<kWide * grid, kCoThreads, 0, st>>>(S, role, off, stg, counts);
     if (passes) {
-        k_co_pairs<<<grid, kCoThreads, 0, st>>>(S, C, vals[cur], runs, role, cs.rsum, off, stg,
+        k_co_pairs<<<kWide * grid, kCoThreads, 0, st>>>(S, C, vals[cur], runs, role, cs.rsum, off, stg,
                                                  counts);
     }
-    k_co_copy_back<<<grid, kCoThreads, 0, st>>>(S, stg, counts, stats);
+    k_co_copy_back<<<kWide * grid, kCoThreads, 0, st>>>(S, stg, counts, stats);
     return cudaGetLastError();
 }
 
@@ -741,7 +830,6 @@ cudaError_t launch_sort_cells(const SpeciesDev &S, const YeeGrid &g, void *scrat
     unsigned long long *const *keys = cs.keys;
     unsigned *const *vals = cs.vals;
     const Stage stg = cs.stg;
-    unsigned *hist = cs.hist;
     long long *counts = cs.counts;
     const unsigned long long top = (unsigned long long)g.nx * (unsigned long long)g.ny;
     int bits = 0;
@@ -749,17 +837,10 @@ cudaError_t launch_sort_cells(const SpeciesDev &S, const YeeGrid &g, void *scrat
     const int passes = (bits + 7) / 8;
     cudaError_t e = cudaMemsetAsync(stats, 0, 4 * 8, st);
     if (e != cudaSuccess) return e;
-    k_sort_prepare<<<grid, kCoThreads, 0, st>>>(S, g, keys[0], vals[0], counts, status);
-    int cur = 0;
-    for (int ps = 0; ps < passes; ++ps) {
-        k_co_hist<<<grid, kCoThreads, 0, st>>>(keys[cur], 8 * ps, hist, counts);
-        k_co_scan<<<1, 1024, 0, st>>>(hist, kRadix * grid, nullptr);
-        k_co_scatter<<<grid, kCoThreads, 0, st>>>(keys[cur], vals[cur], keys[cur ^ 1],
-                                                   vals[cur ^ 1], 8 * ps, hist, counts);
-        cur ^= 1;
-    }
-    k_sort_gather<<<grid, kCoThreads, 0, st>>>(S, vals[cur], stg, counts);
-    k_co_copy_back<<<grid, kCoThreads, 0, st>>>(S, stg, counts, stats);
+    k_sort_prepare<<<kWide * grid, kCoThreads, 0, st>>>(S, g, keys[0], vals[0], counts, status);
+    const int cur = radix_sort(cs, passes, grid, st);
+    k_sort_gather<<<kWide * grid, kCoThreads, 0, st>>>(S, vals[cur], stg, counts);
+    k_co_copy_back<<<kWide * grid, kCoThreads, 0, st>>>(S, stg, counts, stats);
     return cudaGetLastError();
 }
 
@@ -809,16 +890,8 @@ cudaError_t launch_fused_order(const SpeciesDev &Ph, void *scratch, int grid, in
                                long long *win, int *status, cudaStream_t st)
 {
     const CoScratch cs = carve(scratch, Ph.present ? Ph.cap : 0, grid);
-    k_fo_prepare<<<grid, kCoThreads, 0, st>>>(Ph, cs.counts, win, cs.vals[0], status);
-    int cur = 0;
-    for (int ps = 0; ps < (key_bits + 7) / 8; ++ps) {
-        k_co_hist<<<grid, kCoThreads, 0, st>>>(cs.keys[cur], 8 * ps, cs.hist, cs.counts);
-        k_co_scan<<<1, 1024, 0, st>>>(cs.hist, kRadix * grid, nullptr);
-        k_co_scatter<<<grid, kCoThreads, 0, st>>>(cs.keys[cur], cs.vals[cur], cs.keys[cur ^ 1],
-                                                   cs.vals[cur ^ 1], 8 * ps, cs.hist,
-                                                   cs.counts);
-        cur ^= 1;
-    }
+    k_fo_prepare<<<kWide * grid, kCoThreads, 0, st>>>(Ph, cs.counts, win, cs.vals[0], status);
+    radix_sort(cs, (key_bits + 7) / 8, grid, st);
     return cudaGetLastError();
 }
 

@@ -70,6 +70,10 @@ cudaError_t launch_deposit(const SpeciesDev &S, double q, double dt, const YeeGr
 cudaError_t launch_sort_cells(const SpeciesDev &S, const YeeGrid &g, void *scratch, int grid,
                               long long *stats, int *status, cudaStream_t st);
 
+// Blocks per SM that own a chunk of slots in the sorts and scans of
+// qp_coalesce.cu (`grid` below is this times the SMs).
+constexpr int kSortBlocksPerSm = 4;
+
 // Compaction / coalescence of a photon species (qp_coalesce.cu): scratch
 // bytes for `cap` slots and `grid` blocks, and the stream-ordered pipeline
 // (P = NULL: compaction only).  stats: 4 device int64 (groups merged,
