@@ -575,10 +575,10 @@ int qp_compact_photons(qp_ctx *ctx, int32_t handle, qp_coalesce_stats *out, void
  * momentum, chi_mean, hist; equal to within rounding, the partition of the
  * sums differs).  The event counters and `status` are context data and come
  * back as 0.
- * Scratch is a static device array of the library sized for
- * QP_NOALLOC_MAX_TILES tiles of 256 slots (QP_NOALLOC_MAX_SLOTS slots, about
- * 2.4 MB), which every GPU that loads the library holds until the process
- * exits.  A species whose capacity exceeds QP_NOALLOC_MAX_SLOTS is rejected
+ * Scratch is a static device array of the library (about 0.3 MB), which
+ * every GPU that loads the library holds until the process exits.  It serves
+ * up to QP_NOALLOC_MAX_TILES tiles of 256 slots (QP_NOALLOC_MAX_SLOTS
+ * slots).  A species whose capacity exceeds QP_NOALLOC_MAX_SLOTS is rejected
  * with QP_ERR_INVALID_ARG before anything is enqueued.  The call runs on the
  * device that owns `d->n_live` (made current for the call, the caller's
  * current device restored before it returns); `stream` must belong to that

@@ -56,7 +56,9 @@ struct qp_ctx {
     int *d_status = nullptr;
     unsigned long long *d_chain = nullptr;  // lepton chain then photon chain
     size_t chain_words = 0;           // words per chain
-    double *d_diag = nullptr;         // partials + final
+    double *d_diag = nullptr;         // partials of the diagnostics' blocks
+    qp::DiagRead *d_read = nullptr;   // what qp_diagnostics reads
+    qp::DiagRead *h_read = nullptr;   // (pinned)
     double *d_stash = nullptr;        // append records of qp_step launches
     size_t stash_bytes = 0;
     void *d_fuse = nullptr;           // scratch of qp_step_fused
@@ -132,6 +134,8 @@ void release(qp_ctx *c)
     cudaFree(c->d_status);
     cudaFree(c->d_chain);
     cudaFree(c->d_diag);
+    cudaFree(c->d_read);
+    cudaFreeHost(c->h_read);
     cudaFree(c->d_stash);
     cudaFree(c->d_coal);
     cudaFree(c->d_coal_stats);
@@ -330,7 +334,9 @@ int qp_init_tables(const qp_table_params *p, qp_ctx **out_ctx)
     QP_TRY(cudaMemset(c->d_pending, 0, 4 * sizeof(long long)));
     QP_TRY(cudaMalloc(&c->d_status, sizeof(int)));
     QP_TRY(cudaMemset(c->d_status, 0, sizeof(int)));
-    QP_TRY(cudaMalloc(&c->d_diag, (qp::kDiagBlocks + 1) * qp::kDiagWords * sizeof(double)));
+    QP_TRY(cudaMalloc(&c->d_diag, (size_t)qp::kDiagBlocks * qp::kDiagWords * sizeof(double)));
+    QP_TRY(cudaMalloc(&c->d_read, sizeof(qp::DiagRead)));
+    QP_TRY(cudaMallocHost((void **)&c->h_read, sizeof(qp::DiagRead)));
 #undef QP_TRY
     int st = ensure_chain(c, 16);
     if (st != QP_OK) {
@@ -1000,23 +1006,17 @@ int qp_diagnostics(qp_ctx *ctx, int32_t handle, qp_diag *out, void *stream)
     cudaStream_t st = (cudaStream_t)stream;
     const qp_species_desc &d = ctx->species[handle].d;
     qp::SpeciesDev S = species_dev(ctx, handle);
-    double *partials = ctx->d_diag;
-    double *fin = ctx->d_diag + (size_t)qp::kDiagBlocks * qp::kDiagWords;
-    cudaError_t e = qp::launch_diag(S, d.kind == QP_PHOTON, partials, qp::kDiagBlocks, fin, st);
+    const qp::DiagOut o{ctx->d_diag, ctx->d_read, ctx->d_stats + handle, ctx->d_status};
+    cudaError_t e = qp::launch_diag(S, d.kind == QP_PHOTON, o, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(ctx->h_read, ctx->d_read, sizeof(qp::DiagRead),
+                            cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_status(e);
-    double h[qp::kDiagWords];
-    qp::DevStats ds;
-    int64_t n_live = 0;
-    int status = 0;
-    if ((e = cudaMemcpyAsync(h, fin, sizeof(h), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&ds, ctx->d_stats + handle, sizeof(ds), cudaMemcpyDeviceToHost, st)) !=
-            cudaSuccess ||
-        (e = cudaMemcpyAsync(&n_live, d.n_live, sizeof(n_live), cudaMemcpyDeviceToHost, st)) !=
-            cudaSuccess ||
-        (e = cudaMemcpyAsync(&status, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, st)) !=
-            cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
-        return cuda_status(e);
+    const double *h = ctx->h_read->sums;
+    const qp::DevStats &ds = ctx->h_read->stats;
+    const int64_t n_live = ctx->h_read->n_live;
+    const int status = ctx->h_read->status;
     memset(out, 0, sizeof(*out));
     out->n_live = n_live;
     out->n_alive = (int64_t)llround(h[0]);

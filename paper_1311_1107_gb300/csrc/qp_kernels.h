@@ -49,8 +49,23 @@ const void *fused_photons_mixed();
 cudaError_t launch_init_tau(double *tau, int64_t first, int64_t count, int64_t id_base,
                             int64_t id_split, int64_t id_append, uint64_t seed, int species,
                             cudaStream_t st);
-cudaError_t launch_diag(const SpeciesDev &S, int is_photon, double *partials, int nblocks,
-                        double *out, cudaStream_t st);
+// Reduction of a species: partials of up to kDiagBlocks blocks, and what the
+// host reads in one copy (stats and status null: left out).
+constexpr int kDiagBlocks = 512;
+constexpr int kDiagWords = 8 + QP_HIST_BINS;  // scalars + histogram per block
+struct DiagRead {
+    double sums[kDiagWords];
+    DevStats stats;
+    int64_t n_live;
+    int32_t status, pad;
+};
+struct DiagOut {
+    double *partials;
+    DiagRead *out;
+    const DevStats *stats;
+    const int *status;
+};
+cudaError_t launch_diag(const SpeciesDev &S, int is_photon, const DiagOut &o, cudaStream_t st);
 cudaError_t launch_wait_selftest(unsigned long long *words, unsigned spin_limit, int *status,
                                  cudaStream_t st);
 
@@ -90,8 +105,5 @@ struct Pulse2DDev {
 cudaError_t launch_pulse_fill(const Pulse2DDev &p, int64_t nx, int64_t ny, double dx, double dy,
                               double x0, double y0, double t, float *ey, float *bz,
                               cudaStream_t st);
-
-constexpr int kDiagBlocks = 256;
-constexpr int kDiagWords = 8 + QP_HIST_BINS;  // scalars + histogram per block
 
 }  // namespace qp

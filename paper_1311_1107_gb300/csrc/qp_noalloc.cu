@@ -11,8 +11,10 @@
 
 namespace {
 
-// One partial row per 256-slot tile, then the final row.
-constexpr size_t kScratchWords = (size_t)(QP_NOALLOC_MAX_TILES + 1) * qp::kDiagWords;
+// The blocks' partial rows, then what the host reads.
+constexpr size_t kPartialWords = (size_t)qp::kDiagBlocks * qp::kDiagWords;
+constexpr size_t kScratchWords = kPartialWords + sizeof(qp::DiagRead) / sizeof(double);
+static_assert(sizeof(qp::DiagRead) % sizeof(double) == 0, "scratch is in words");
 static __device__ __align__(256) double g_noalloc_scratch[kScratchWords];
 
 // Device address of the array, looked up once per device with that device
@@ -101,23 +103,17 @@ extern "C" int qp_diagnostics_noalloc(const qp_species_desc *d, qp_diag *out, vo
     S.n_live = d->n_live;
     S.cap = d->capacity;
     S.present = 1;
-    // one block per tile: every partial row read by the final pass is
-    // written by this call (tiles past the live count write zeros)
-    int tiles = (int)((d->capacity + qp::kDiagTile - 1) / qp::kDiagTile);
-    if (tiles < 1) tiles = 1;
-    double *partials = scratch;
-    double *fin = scratch + (size_t)QP_NOALLOC_MAX_TILES * qp::kDiagWords;
+    qp::DiagRead *read = (qp::DiagRead *)(scratch + kPartialWords);
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = qp::launch_diag(S, d->kind == QP_PHOTON, partials, tiles, fin, s);
-    double h[qp::kDiagWords];
-    int64_t n_live = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h, fin, sizeof(h), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&n_live, d->n_live, sizeof(n_live), cudaMemcpyDeviceToHost, s);
+    cudaError_t e = qp::launch_diag(S, d->kind == QP_PHOTON,
+                                    qp::DiagOut{scratch, read, nullptr, nullptr}, s);
+    qp::DiagRead r;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&r, read, sizeof(r), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? QP_ERR_OOM : QP_ERR_CUDA;
+    const double *h = r.sums;
     memset(out, 0, sizeof(*out));
-    out->n_live = n_live;
+    out->n_live = r.n_live;
     out->n_alive = (int64_t)llround(h[0]);
     out->weight = h[1];
     out->energy = h[2];
