@@ -463,8 +463,16 @@ int qp_fill_yee2d(qp_ctx *ctx, const qp_pulse2d *p, const qp_field *grid, double
  *   J = 0; qp_deposit_current for electrons and positrons: J^(n+1/2)
  *   qp_yee_advance_b(dt/2)   B^n -> B^(n+1/2)
  *   qp_yee_advance_e(dt, J)  E^n -> E^(n+1)
+ * qp_pic_step runs whole cycles.
  * QP_ERR_INVALID_ARG for a grid of another kind or with a missing component.
  */
+
+/* s->n_steps cycles as above on the grid s->field with time step s->dt; jx,
+ * jy, jz: device float arrays of ny rows of nx values on E's staggering, left
+ * with the last cycle's current.  Five launches a cycle: J is zeroed by the
+ * first B half step, both lepton species are deposited together. */
+int qp_pic_step(qp_ctx *ctx, const qp_step_params *s, float *jx, float *jy, float *jz,
+                void *stream);
 
 /* B -= dtb curl E on the grid, in place. */
 int qp_yee_advance_b(qp_ctx *ctx, const qp_field *grid, double dtb, void *stream);

@@ -60,6 +60,7 @@ struct qp_ctx {
     qp::DiagRead *d_read = nullptr;   // what qp_diagnostics reads
     qp::DiagRead *h_read = nullptr;   // (pinned)
     double *d_stash = nullptr;        // append records of qp_step launches
+    std::vector<double *> old_stash;  // outgrown ones
     size_t stash_bytes = 0;
     void *d_fuse = nullptr;           // scratch of qp_step_fused
     size_t fuse_bytes = 0;
@@ -137,6 +138,7 @@ void release(qp_ctx *c)
     cudaFree(c->d_read);
     cudaFreeHost(c->h_read);
     cudaFree(c->d_stash);
+    for (double *p : c->old_stash) cudaFree(p);
     cudaFree(c->d_coal);
     cudaFree(c->d_coal_stats);
     cudaFree(c->d_fuse);
@@ -743,13 +745,16 @@ int qp_step(qp_ctx *ctx, const qp_step_params *s, void *stream)
     const int grid = (int)(cap_tiles < resident ? (cap_tiles > 0 ? cap_tiles : 1) : resident);
     const bool long_ok = qp::has_long_tiles(s->field.kind) &&
                          qp::long_tiles(cap_tiles * qp::kWarps, grid);
-    const size_t stash = (size_t)grid * qp::stash_words(long_ok) * sizeof(double);
+    // For the resident blocks, whatever the grid, so that it grows a few times
+    // at most: with the precision and when long tiles are first met.  A stash
+    // that was outgrown stays until the context goes: a captured step may hold it.
+    const size_t stash = (size_t)resident * qp::stash_words(long_ok) * sizeof(double);
     if (stash > ctx->stash_bytes) {
         // grows (an allocation, synchronous)
         double *p = nullptr;
         cudaError_t e = cudaMalloc(&p, stash);
         if (e != cudaSuccess) return cuda_status(e);
-        cudaFree(ctx->d_stash);
+        if (ctx->d_stash) ctx->old_stash.push_back(ctx->d_stash);
         ctx->d_stash = p;
         ctx->stash_bytes = stash;
     }
@@ -1152,7 +1157,7 @@ int qp_yee_advance_b(qp_ctx *ctx, const qp_field *grid, double dtb, void *stream
     if (!yee_grid_of(grid, g) || !isfinite(dtb)) return QP_ERR_INVALID_ARG;
     DeviceGuard d(ctx->device);
     if (!d.ok) return QP_ERR_CUDA;
-    return cuda_status(qp::launch_yee_b(g, dtb, ctx->num_sms, (cudaStream_t)stream));
+    return cuda_status(qp::launch_yee_b(g, dtb, nullptr, ctx->num_sms, (cudaStream_t)stream));
 }
 
 int qp_yee_advance_e(qp_ctx *ctx, const qp_field *grid, const float *jx, const float *jy,
@@ -1178,8 +1183,54 @@ int qp_deposit_current(qp_ctx *ctx, int32_t handle, const qp_field *grid, float 
     DeviceGuard d(ctx->device);
     if (!d.ok) return QP_ERR_CUDA;
     const double q = sd.kind == QP_ELECTRON ? -1.0 : 1.0;
-    return cuda_status(qp::launch_deposit(species_dev(ctx, handle), q, dt, g, jx, jy, jz,
+    return cuda_status(qp::launch_deposit(species_dev(ctx, handle), q, qp::SpeciesDev{}, 0.0, dt, g, jx, jy, jz,
                                           ctx->d_status, ctx->num_sms, (cudaStream_t)stream));
+}
+
+// A cycle is a chain of short launches (5 us a field update, 39 us the step),
+// each 2 us after the one before: five of them, where the calls one by one are
+// seven with the zeroing of J (eight cycles of a 2048 x 511 grid: 782 -> 722 us).
+int qp_pic_step(qp_ctx *ctx, const qp_step_params *s, float *jx, float *jy, float *jz,
+                void *stream)
+{
+    if (!ctx) return QP_ERR_NOT_INITIALIZED;
+    if (!s || !jx || !jy || !jz || s->n_steps < 0 || !isfinite(s->dt)) return QP_ERR_INVALID_ARG;
+    qp::YeeGrid g{};
+    if (!yee_grid_of(&s->field, g)) return QP_ERR_INVALID_ARG;
+    // the leptons that there are
+    qp::SpeciesDev lep[2] = {};
+    double q[2] = {0.0, 0.0};
+    int n_lep = 0;
+    const int32_t hs[2] = {s->electron, s->positron};
+    for (int k = 0; k < 2; ++k) {
+        if (hs[k] == -1) continue;
+        if (!valid_handle(ctx, hs[k])) return QP_ERR_NOT_INITIALIZED;
+        if (ctx->species[hs[k]].d.capacity == 0) continue;
+        lep[n_lep] = species_dev(ctx, hs[k]);
+        q[n_lep++] = k == 0 ? -1.0 : 1.0;
+    }
+    DeviceGuard d(ctx->device);
+    if (!d.ok) return QP_ERR_CUDA;
+    cudaStream_t cs = (cudaStream_t)stream;
+    float *const j[3] = {jx, jy, jz};
+    qp_step_params one = *s;
+    one.n_steps = 1;
+    for (int32_t k = 0; k < s->n_steps; ++k) {
+        one.step = s->step + k;
+        cudaError_t e = qp::launch_yee_b(g, 0.5 * s->dt, j, ctx->num_sms, cs);
+        if (e != cudaSuccess) return cuda_status(e);
+        const int st = qp_step(ctx, &one, stream);
+        if (st != QP_OK) return st;
+        if (n_lep) {
+            e = qp::launch_deposit(lep[0], q[0], lep[1], q[1], s->dt, g, jx, jy, jz,
+                                   ctx->d_status, ctx->num_sms, cs);
+            if (e != cudaSuccess) return cuda_status(e);
+        }
+        e = qp::launch_yee_b(g, 0.5 * s->dt, nullptr, ctx->num_sms, cs);
+        if (e == cudaSuccess) e = qp::launch_yee_e(g, jx, jy, jz, s->dt, ctx->num_sms, cs);
+        if (e != cudaSuccess) return cuda_status(e);
+    }
+    return QP_OK;
 }
 
 int qp_sort_species(qp_ctx *ctx, int32_t handle, const qp_field *grid, void *stream)

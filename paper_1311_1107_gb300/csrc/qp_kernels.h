@@ -75,11 +75,14 @@ struct YeeGrid {
     int64_t nx, ny;
     double dx, dy, x0, y0;
 };
-cudaError_t launch_yee_b(const YeeGrid &g, double dtb, int num_sms, cudaStream_t st);
+// j: the current's three arrays, zeroed in the same pass, or null.
+cudaError_t launch_yee_b(const YeeGrid &g, double dtb, float *const *j, int num_sms,
+                         cudaStream_t st);
 cudaError_t launch_yee_e(const YeeGrid &g, const float *jx, const float *jy, const float *jz,
                          double dt, int num_sms, cudaStream_t st);
-cudaError_t launch_deposit(const SpeciesDev &S, double q, double dt, const YeeGrid &g, float *jx,
-                           float *jy, float *jz, int *status, int num_sms, cudaStream_t st);
+// The currents of A and, if present, of B.
+cudaError_t launch_deposit(const SpeciesDev &A, double q_a, const SpeciesDev &B, double q_b,
+                           double dt, const YeeGrid &g, float *jx, float *jy, float *jz, int *status, int num_sms, cudaStream_t st);
 // Stable sort of a species' live slots by cell of g (qp_coalesce.cu; the
 // coalescence scratch, stats as there).
 cudaError_t launch_sort_cells(const SpeciesDev &S, const YeeGrid &g, void *scratch, int grid,

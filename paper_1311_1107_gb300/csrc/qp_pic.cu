@@ -28,7 +28,13 @@ __device__ __forceinline__ float at(const float *a, int64_t nx, int64_t ny, int6
 
 // Nodes by rows: blockIdx.y strides over the rows, the threads of blockIdx.x
 // over the columns (no index division).
-__global__ void __launch_bounds__(kPicBlock) k_yee_b(YeeGrid g, float idx, float idy, float dtb)
+// clear: the current's three arrays, set to 0 on the way, or null.
+struct Clear {
+    float *j[3];
+};
+
+__global__ void __launch_bounds__(kPicBlock) k_yee_b(YeeGrid g, float idx, float idy, float dtb,
+                                                     Clear clear)
 {
     for (int64_t j = blockIdx.y; j < g.ny; j += gridDim.y)
         for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < g.nx;
@@ -42,6 +48,7 @@ __global__ void __launch_bounds__(kPicBlock) k_yee_b(YeeGrid g, float idx, float
             g.f[3][k] -= dtb * dEz_dy;
             g.f[4][k] += dtb * dEz_dx;
             g.f[5][k] -= dtb * (dEy_dx - dEx_dy);
+            if (clear.j[0]) clear.j[0][k] = clear.j[1][k] = clear.j[2][k] = 0.0f;
         }
 }
 
@@ -74,7 +81,8 @@ __device__ __forceinline__ float4 ld4(const float *a, int64_t k)
     return *reinterpret_cast<const float4 *>(a + k);
 }
 
-__global__ void __launch_bounds__(kPicBlock) k_yee_b4(YeeGrid g, float idx, float idy, float dtb)
+__global__ void __launch_bounds__(kPicBlock) k_yee_b4(YeeGrid g, float idx, float idy, float dtb,
+                                                      Clear clear)
 {
     const int64_t nq = g.nx / 4;
     for (int64_t j = blockIdx.y; j < g.ny; j += gridDim.y)
@@ -105,6 +113,10 @@ __global__ void __launch_bounds__(kPicBlock) k_yee_b4(YeeGrid g, float idx, floa
             *reinterpret_cast<float4 *>(g.f[3] + k) = bx;
             *reinterpret_cast<float4 *>(g.f[4] + k) = by;
             *reinterpret_cast<float4 *>(g.f[5] + k) = bz;
+            if (clear.j[0])
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    *reinterpret_cast<float4 *>(clear.j[c] + k) = make_float4(0.f, 0.f, 0.f, 0.f);
         }
 }
 
@@ -156,7 +168,6 @@ __global__ void __launch_bounds__(kPicBlock) k_yee_e4(YeeGrid g, float idx, floa
 // x0/dx, y0/dy as float pairs (hi + lo) so that the cell coordinate of a
 // position keeps double-float precision without an FP64 instruction.
 struct DepositConsts {
-    float q_area;                    // q / (dx dy)
     float idx_hi, idx_lo, idy_hi, idy_lo;
     float x0s_hi, x0s_lo, y0s_hi, y0s_lo;
     float hdt_x, hdt_y;              // dt / (2 dx), dt / (2 dy)
@@ -184,19 +195,26 @@ __device__ __forceinline__ float cell_of(df2 a, float &frac)
 // component's staggered nodes (Jx at i+1/2, Jy at j+1/2, Jz at the node).
 // The FP64 state is read as double-float positions and nearest-float
 // momenta and weights by integer instructions (qp_df.h): no instruction
-// runs on the FP64 pipe.
-__global__ void __launch_bounds__(kPicBlock) k_deposit(SpeciesDev S, DepositConsts c, YeeGrid g,
-                                                       float *jx, float *jy, float *jz,
+// runs on the FP64 pipe.  Two species a launch: the first `blocks_a` blocks
+// take A, the others B.
+__global__ void __launch_bounds__(kPicBlock) k_deposit(SpeciesDev A, SpeciesDev B, int blocks_a,
+                                                       float q_a, float q_b, DepositConsts c,
+                                                       YeeGrid g, float *jx, float *jy, float *jz,
                                                        int *status)
 {
+    const bool first = (int)blockIdx.x < blocks_a;
+    const SpeciesDev &S = first ? A : B;
+    const int block = first ? blockIdx.x : blockIdx.x - blocks_a;
+    const int blocks = first ? blocks_a : gridDim.x - blocks_a;
+    const float q_area = first ? q_a : q_b;
     long long n = *((volatile long long *)S.n_live);
     if (n < 0 || n > S.cap) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) raise_status(status, QP_ERR_INVALID_ARG);
+        if (block == 0 && threadIdx.x == 0) raise_status(status, QP_ERR_INVALID_ARG);
         n = n < 0 ? 0 : S.cap;
     }
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t stride = (int64_t)blocks * blockDim.x;
     float *J[3] = {jx, jy, jz};
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += stride) {
+    for (int64_t p = (int64_t)block * blockDim.x + threadIdx.x; p < n; p += stride) {
         const double xd = S.x[p], yd = S.y[p], uxd = S.ux[p], uyd = S.uy[p], uzd = S.uz[p],
                      wd = S.w[p];
         const float ux = hi_d(uxd), uy = hi_d(uyd), uz = hi_d(uzd);
@@ -209,7 +227,7 @@ __global__ void __launch_bounds__(kPicBlock) k_deposit(SpeciesDev S, DepositCons
         const df2 gy = df_add_f(df_sub(df_mul(split_d(yd), {c.idy_hi, c.idy_lo}),
                                        {c.y0s_hi, c.y0s_lo}),
                                 -c.hdt_y * v[1]);
-        const float a = c.q_area * hi_d(wd);
+        const float a = q_area * hi_d(wd);
         float fx0, fy0, fxh, fyh;
         const float fi0 = cell_of(gx, fx0), fj0 = cell_of(gy, fy0);
         const float fih = cell_of(df_add_f(gx, -0.5f), fxh), fjh = cell_of(df_add_f(gy, -0.5f), fyh);
@@ -277,14 +295,16 @@ int grid_blocks(int64_t n, int num_sms)
 
 }  // namespace
 
-cudaError_t launch_yee_b(const YeeGrid &g, double dtb, int num_sms, cudaStream_t st)
+cudaError_t launch_yee_b(const YeeGrid &g, double dtb, float *const *j, int num_sms,
+                         cudaStream_t st)
 {
+    const Clear clear = j ? Clear{{j[0], j[1], j[2]}} : Clear{{nullptr, nullptr, nullptr}};
     // 1/dx and 1/dy once, as each node would form them (FP64 quotient to float)
     const float idx = (float)(1.0 / g.dx), idy = (float)(1.0 / g.dy);
-    if (quads(g))
-        k_yee_b4<<<quad_grid(g, num_sms), kPicBlock, 0, st>>>(g, idx, idy, (float)dtb);
+    if (quads(g, clear.j[0], clear.j[1], clear.j[2]))
+        k_yee_b4<<<quad_grid(g, num_sms), kPicBlock, 0, st>>>(g, idx, idy, (float)dtb, clear);
     else
-        k_yee_b<<<node_grid(g, num_sms), kPicBlock, 0, st>>>(g, idx, idy, (float)dtb);
+        k_yee_b<<<node_grid(g, num_sms), kPicBlock, 0, st>>>(g, idx, idy, (float)dtb, clear);
     return cudaGetLastError();
 }
 
@@ -301,8 +321,9 @@ cudaError_t launch_yee_e(const YeeGrid &g, const float *jx, const float *jy, con
     return cudaGetLastError();
 }
 
-cudaError_t launch_deposit(const SpeciesDev &S, double q, double dt, const YeeGrid &g, float *jx,
-                           float *jy, float *jz, int *status, int num_sms, cudaStream_t st)
+cudaError_t launch_deposit(const SpeciesDev &A, double q_a, const SpeciesDev &B, double q_b,
+                           double dt, const YeeGrid &g, float *jx, float *jy, float *jz,
+                           int *status, int num_sms, cudaStream_t st)
 {
     DepositConsts c;
     const double idx = 1.0 / g.dx, idy = 1.0 / g.dy, x0s = g.x0 * idx, y0s = g.y0 * idy;
@@ -310,14 +331,18 @@ cudaError_t launch_deposit(const SpeciesDev &S, double q, double dt, const YeeGr
         hi = (float)v;
         lo = (float)(v - (double)hi);
     };
-    c.q_area = (float)(q / (g.dx * g.dy));
     split(idx, c.idx_hi, c.idx_lo);
     split(idy, c.idy_hi, c.idy_lo);
     split(x0s, c.x0s_hi, c.x0s_lo);
     split(y0s, c.y0s_hi, c.y0s_lo);
     c.hdt_x = (float)(0.5 * dt * idx);
     c.hdt_y = (float)(0.5 * dt * idy);
-    k_deposit<<<grid_blocks(S.cap, num_sms), kPicBlock, 0, st>>>(S, c, g, jx, jy, jz, status);
+    const double area = g.dx * g.dy;
+    const int blocks_a = grid_blocks(A.cap, num_sms);
+    const int blocks_b = B.present ? grid_blocks(B.cap, num_sms) : 0;
+    k_deposit<<<blocks_a + blocks_b, kPicBlock, 0, st>>>(A, B, blocks_a, (float)(q_a / area),
+                                                         (float)(q_b / area), c, g, jx, jy, jz,
+                                                         status);
     return cudaGetLastError();
 }
 

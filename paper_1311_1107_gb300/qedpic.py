@@ -131,7 +131,7 @@ EXPORTS = ("qp_init_tables", "qp_destroy", "qp_create_species", "qp_init_optical
            "qp_batch_create", "qp_batch_destroy", "qp_batch_scratch_words", "qp_batch_set",
            "qp_batch_clear", "qp_batch_step", "qp_batch_progress", "qp_coalesce_photons",
            "qp_compact_photons", "qp_fill_yee2d", "qp_step_fused", "qp_yee_advance_b",
-           "qp_yee_advance_e", "qp_deposit_current", "qp_sort_species")
+           "qp_yee_advance_e", "qp_deposit_current", "qp_sort_species", "qp_pic_step")
 
 
 def library_path() -> str:
@@ -183,6 +183,7 @@ def lib(build_if_missing: bool = False):
         L.qp_yee_advance_e.argtypes = [vp, C.POINTER(qp_field), vp, vp, vp, C.c_double, vp]
         L.qp_deposit_current.argtypes = [vp, i32, C.POINTER(qp_field), vp, vp, vp, C.c_double,
                                          vp]
+        L.qp_pic_step.argtypes = [vp, C.POINTER(qp_step_params), vp, vp, vp, vp]
         L.qp_sort_species.argtypes = [vp, i32, C.POINTER(qp_field), vp]
         L.qp_fill_yee2d.argtypes = [vp, C.POINTER(qp_pulse2d), C.POINTER(qp_field), C.c_double,
                                     vp]
@@ -411,6 +412,11 @@ def qp_deposit_current(ctx, handle: int, grid: qp_field, jx_ptr, jy_ptr, jz_ptr,
     return _check("qp_deposit_current",
                   lib().qp_deposit_current(ctx, handle, C.byref(grid), jx_ptr, jy_ptr, jz_ptr,
                                            float(dt), stream))
+
+
+def qp_pic_step(ctx, params: qp_step_params, jx_ptr, jy_ptr, jz_ptr, stream=None) -> int:
+    return _check("qp_pic_step", lib().qp_pic_step(ctx, C.byref(params), jx_ptr, jy_ptr, jz_ptr,
+                                                   stream))
 
 
 def qp_sort_species(ctx, handle: int, grid: qp_field, stream=None) -> int:

@@ -203,31 +203,14 @@ class Simulation:
         self.step_index += int(n_steps)
         return st
 
-    def _pic_step(self, sh) -> int:
-        """One PIC cycle: B half step, the QED step, the current, B half
-        step, E full step (E^n and B^(n-1/2) stored between cycles)."""
-        dt = self.params.dt
-        Q.qp_yee_advance_b(self.ctx, self.field, 0.5 * dt, sh)
-        self.params.step = self.step_index
-        self.params.n_steps = 1
-        st = Q.qp_step(self.ctx, self.params, sh)
-        self.J.zero_()
-        j = [self.J[k].data_ptr() for k in range(3)]
-        for name in ("electron", "positron"):
-            sp = self.species[name]
-            if sp.cap > 0:
-                Q.qp_deposit_current(self.ctx, sp.handle, self.field, j[0], j[1], j[2], dt, sh)
-        Q.qp_yee_advance_b(self.ctx, self.field, 0.5 * dt, sh)
-        Q.qp_yee_advance_e(self.ctx, self.field, j[0], j[1], j[2], dt, sh)
-        self.step_index += 1
-        return st
-
     def run(self, n_steps: int, stream=None) -> int:
         if self.pic_pulse is not None:
-            sh = stream_handle(stream)
-            st = 0
-            for _ in range(int(n_steps)):
-                st = max(st, self._pic_step(sh))
+            # PIC cycles (E^n and B^(n-1/2) stored between cycles)
+            self.params.step = self.step_index
+            self.params.n_steps = int(n_steps)
+            j = [self.J[k].data_ptr() for k in range(3)]
+            st = Q.qp_pic_step(self.ctx, self.params, j[0], j[1], j[2], stream_handle(stream))
+            self.step_index += int(n_steps)
             return st
         if self.pulse is not None:
             # fields refilled from the pulse at each step's time, then the step
