@@ -280,4 +280,79 @@ QP_HD double add_fd(double d, float f)
     return add_fd_wide(d, f);
 }
 
+// ------------------------------------------------------------------ equal steps
+
+// The increments that repeat_step takes: sum(x) is x and the exact increment
+// rounded once, one(x) the step as it is defined, equal to sum(x) where
+// exact(e) holds for x's biased exponent e and sum(x) has that exponent too;
+// rest(D) is the increment less D, rounded.
+struct StepFloat {  // add_fd(x, f)
+    double d;
+    float f;
+    QP_HD explicit StepFloat(float f_) : d(f_to_d(f_)), f(f_) {}
+    QP_HD double one(double x) const { return add_fd(x, f); }
+    QP_HD double sum(double x) const { return x + d; }
+    QP_HD double rest(double D) const { return d - D; }
+    QP_HD bool exact(int e) const { return (int)((f2u(f) >> 23) & 0xFFu) - e + 925 <= 28; }
+};
+struct StepProduct {  // fma(a, b, x)
+    double a, b;
+    QP_HD double one(double x) const { return fma(a, b, x); }
+    QP_HD double sum(double x) const { return fma(a, b, x); }
+    QP_HD double rest(double D) const { return fma(a, b, -D); }
+    QP_HD bool exact(int) const { return true; }
+};
+
+// x after n equal steps: the bits of taking them one by one.  While x keeps its
+// exponent its values lie on one grid, so every step that is no tie rounds to
+// the same difference D (exact), and k of them are x + k D, exact as well: one
+// addition a binade crossed, not one a step.  k keeps clear of the binade's end
+// by an FP32 estimate; the sum is taken only if it stays inside, and a step
+// otherwise.  (A fused window's photons move up to its length, each step an
+// instruction of the FP64 pipe and coordinate: 250 steps of 4096 electrons
+// 1570 -> 1469 us.)
+template <class Step>
+QP_HD double repeat_step(double x, int n, const Step &s)
+{
+    while (n > 0) {
+        const uint64_t bx = d2u(x);
+        const int e = (int)(bx >> 52) & 0x7FF;
+        const double y = s.sum(x);
+        const uint64_t by = d2u(y);
+        bool stepped = false;
+        if (n > 3 && e >= 960 && e < 1150 && s.exact(e) && (by >> 52) == (bx >> 52)) {
+            if (by == bx) return x;
+            const double D = y - x;
+            if ((d2u(s.rest(D)) << 1 >> 1) == (uint64_t)(e - 53) << 52) {  // ties: parity decides
+                for (; n > 0; --n) x = s.one(x);
+                return x;
+            }
+            const uint64_t mant = bx & 0xFFFFFFFFFFFFFull;
+            const bool inward = ((d2u(D) ^ bx) >> 63) != 0u;
+            const uint32_t room = (uint32_t)((inward ? mant : 0xFFFFFFFFFFFFFull - mant) >> 20);
+            // room 2^20 units of the last place, 2^(e - 1055), over |D|
+            const float q = (float)room * u2f((uint32_t)(e - 928) << 23) /
+                            u2f(f2u(hi_d(D)) & 0x7FFFFFFFu);
+            const float c = q * 0.99999f - 1.0f;
+            if (c >= 2.0f) {
+                const int k = c < (float)n ? (int)c : n;
+                const double t = fma(k < (1 << 24) ? f_to_d((float)k) : (double)k, D, x);
+                const uint64_t bt = d2u(t);
+                if ((bt >> 52) == (bx >> 52) && (bt << 12) != 0u) {
+                    x = t;
+                    n -= k;
+                    stepped = true;
+                }
+            }
+        }
+        if (!stepped) {
+            const double z = s.one(x);
+            if (d2u(z) == bx) return x;
+            x = z;
+            --n;
+        }
+    }
+    return x;
+}
+
 }  // namespace qp

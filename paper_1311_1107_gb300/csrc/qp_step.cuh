@@ -2455,22 +2455,18 @@ __global__ void __launch_bounds__(256) k_fused_photons(const __grid_constant__ F
                 const double u2 = photon_u64(ux, uy, uz);
                 if (u2 > 0.0) {
                     const double ig = rsqrt64(u2);
-                    for (int m = 0; m < moves; ++m) {
-                        x = photon_move64(x, ux, ig, P.dt);
-                        y = photon_move64(y, uy, ig, P.dt);
-                        z = photon_move64(z, uz, ig, P.dt);
-                    }
+                    x = repeat_step(x, moves, StepProduct{P.dt, __dmul_rn(ux, ig)});
+                    y = repeat_step(y, moves, StepProduct{P.dt, __dmul_rn(uy, ig)});
+                    z = repeat_step(z, moves, StepProduct{P.dt, __dmul_rn(uz, ig)});
                 }
             } else {
                 const float fx = hi_d(ux), fy = hi_d(uy), fz = hi_d(uz);
                 const float g = photon_speed32(fx, fy, fz);
                 if (g > 0.0f) {
                     const float c = P.mc.dt / g;
-                    for (int m = 0; m < moves; ++m) {
-                        x = photon_move32(x, fx, c);
-                        y = photon_move32(y, fy, c);
-                        z = photon_move32(z, fz, c);
-                    }
+                    x = repeat_step(x, moves, StepFloat(c * fx));
+                    y = repeat_step(y, moves, StepFloat(c * fy));
+                    z = repeat_step(z, moves, StepFloat(c * fz));
                 }
             }
         }
