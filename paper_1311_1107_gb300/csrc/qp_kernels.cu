@@ -245,6 +245,21 @@ int fused_key_bits(int K, long long tiles, int *ordinal_bits)
     return bits_of((unsigned long long)(K > 1 ? K - 1 : 0)) + ob + kEmitBits;
 }
 
+// Warps an SM up to which a fused window's tiles of 32 leptons are split into
+// warps of fewer lanes.  A window is a chain of K steps a warp, each as long as
+// the emission loops of its slowest lane, and a few thousand leptons leave most
+// of the chip idle: fewer lanes a warp meet fewer of them.  On the FP64 path a
+// warp's instruction takes the pipe 20 cycles however few its lanes, so the
+// line lies lower.  Measured, us a window, whole tiles and split up to 2 / 4 /
+// 8 / 16 warps an SM:
+//   mixed  4096 leptons x 250 steps 1519: 1265 / 1024 /  935 /  988
+//          9000 x 100                723:  714 /  631 /  564 /  585
+//         20000 x 100                793:  787 /  792 /  788 /  739
+//   FP64   1500 x 200               3011: 2083 / 1755 / 1814 / 1809
+//          4096 x 250               3811: 3263 / 2655 / 3235 / 5222
+//          9000 x 100               1638: 1634 / 1500 / 1871 / 2724
+constexpr int kFusedWarpsMixed = 8, kFusedWarpsFp64 = 4;
+
 cudaError_t launch_fused(const StepArgs &a, int precision, int field_kind, int K,
                          long long tiles_e, long long tiles, void *scratch, int order_grid,
                          long long *win, int num_sms, cudaStream_t st)
@@ -264,7 +279,10 @@ cudaError_t launch_fused(const StepArgs &a, int precision, int field_kind, int K
     f.win = win;
     void *args[] = {(void *)&f};
     const long long resident = (long long)num_sms * 32;
-    const unsigned grid = (unsigned)(tiles < resident ? (tiles > 0 ? tiles : 1) : resident);
+    const int most = mixed ? kFusedWarpsMixed : kFusedWarpsFp64;
+    while (f.split < 5 && (tiles << (f.split + 1)) <= (long long)most * num_sms) ++f.split;
+    const long long warps = tiles << f.split;
+    const unsigned grid = (unsigned)(warps < resident ? (warps > 0 ? warps : 1) : resident);
     cudaError_t e = cudaMemsetAsync(f.fs.alloc, 0, sizeof(long long), st);
     if (e == cudaSuccess) e = cudaLaunchKernel(lep, dim3(grid), dim3(32), args, 0, st);
     if (e == cudaSuccess) e = launch_fused_order(Ph, scratch, order_grid, key_bits, win, a.status, st);

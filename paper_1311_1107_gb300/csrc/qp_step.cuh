@@ -2197,7 +2197,8 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
 // and step) and are staged there with their order key: step, then emitter
 // (tile, lane), then emission index, the slot order of K separate steps.
 // The key sort (launch_fused_order) and k_fused_photons put them at those
-// slots.  Tiles are one warp.
+// slots.  A tile of 32 leptons is one warp, or several of fewer lanes where
+// the leptons leave the chip idle (launch_fused).
 
 constexpr int kEmitBits = 3;
 static_assert(QP_MAX_EMISSIONS <= (1 << kEmitBits), "emission index bits");
@@ -2206,7 +2207,8 @@ struct FusedArgs {
     StepArgs a;              // a.single: the problem at the window's first step
     int32_t K;               // steps in the window
     int32_t ob;              // bits of the emitter ordinal (tile * 32 + lane) in the key
-    long long tiles_e, tiles; // lepton tiles (electron tiles first)
+    long long tiles_e, tiles; // lepton tiles of 32 slots (electron tiles first)
+    int32_t split;           // a tile is 2^split warps of 32 / 2^split lanes
     FusedScratch fs;
     long long *win;          // [3] photons at the window start, stored and staged in it
 };
@@ -2282,7 +2284,10 @@ __global__ void __launch_bounds__(32, 32) k_fused(const __grid_constant__ FusedA
         }
         if (blockIdx.x == 0 && lane == 0) f.win[0] = base;
     }
-    for (long long tile = blockIdx.x; tile < f.tiles; tile += gridDim.x) {
+    const int lanes = 32 >> f.split;
+    for (long long t = blockIdx.x; t < f.tiles << f.split; t += gridDim.x) {
+        const long long tile = t >> f.split;
+        const int first_lane = lanes * (int)(t & ((1 << f.split) - 1));
         {
             const int *src = reinterpret_cast<const int *>(&a.single);
             int *dst = reinterpret_cast<int *>(&sP);
@@ -2292,20 +2297,21 @@ __global__ void __launch_bounds__(32, 32) k_fused(const __grid_constant__ FusedA
         __syncwarp();
         const int sp = tile < f.tiles_e ? 0 : 1;
         const SpeciesDev &S = sP.sp[sp];
-        const int64_t i = (tile - (sp ? f.tiles_e : 0)) * 32 + lane;
+        const int64_t i = (tile - (sp ? f.tiles_e : 0)) * 32 + first_lane + lane;
         long long n = *((volatile long long *)S.n_live);
         if (n < 0 || n > S.cap) {
             if (lane == 0) raise_status(a.status, QP_ERR_INVALID_ARG);
             n = n < 0 ? 0 : S.cap;
         }
-        const bool active = i < n;
+        const bool active = lane < lanes && i < n;
         LeptonState cur{};
         double w = 0.0;
         if (active) {
             cur = {S.x[i], S.y[i], S.z ? S.z[i] : 0.0, S.ux[i], S.uy[i], S.uz[i], S.tau[i]};
             w = S.w[i];
         }
-        const unsigned long long ordinal = (unsigned long long)(tile * 32 + lane) << kEmitBits;
+        const unsigned long long ordinal = (unsigned long long)(tile * 32 + first_lane + lane)
+                                           << kEmitBits;
         const uint64_t s0 = sP.step;
         unsigned c_emit = 0, c_sub = 0, c_cont = 0, c_sat = 0, c_clamp = 0, c_ph = 0, c_drop = 0;
         double e_sub = 0.0, e_drop = 0.0, chi_last = 0.0;
