@@ -96,9 +96,13 @@ struct StepTime {
 // kDoneGroups group counters (one 32-byte sector each) and the last of each
 // group in `done`: no counter sees more than a few tens of atomics at once.
 constexpr int kDoneGroups = 32;
+// The spread of a launch's first tiles (spread_ticket): blocks met on each SM
+// (SM ids modulo kSpreadSms) and as each SM's n-th, and blocks counted.
+constexpr int kSpreadSms = 256, kSpreadRanks = 32;
 struct StepCtl {
-    unsigned ticket, done, epoch, pad;
+    unsigned ticket, done, epoch, arrived;
     unsigned grp[kDoneGroups][8];
+    unsigned sm_blocks[kSpreadSms], rank_blocks[kSpreadRanks];
 };
 
 constexpr int kMaxProblems = 64;  // problems (independent runs) per launch

@@ -93,6 +93,37 @@ __device__ __noinline__ bool await_epoch(const unsigned *p, unsigned epoch, unsi
     return true;
 }
 
+// The first ticket of a block of a cooperative launch of several steps: 0 ..
+// grid - 1, those of the blocks that came first on their SM before those that
+// came second, and so on.  Blocks that follow one another share an SM, and so
+// did the few tiles of a small step, whose warps then queue for one SM's pipes.
+// Us for 20 steps of a plane wave, block b taking tile b / this:
+//   FP64   4096 electrons 1124 / 761, 8000 1131 / 821, 20000 1135 / 970, a
+//          cascade of 16384 with diagnostics 1554 / 1441;
+//   mixed  4096 458 / 424, 8000 556 / 472, 20000 and 40000 photons 570 / 510.
+// One thread a block; every block is resident, so the wait for all of them ends
+// (it is bounded; no tile and the status on a time-out).  It costs some 2 us, so
+// a launch of one step does without.
+__device__ __noinline__ long long spread_ticket(StepCtl *ctl, unsigned limit, int *status)
+{
+    unsigned sm;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+    const unsigned seen = atomicAdd(&ctl->sm_blocks[sm % kSpreadSms], 1u);
+    const unsigned rank = seen < kSpreadRanks ? seen : kSpreadRanks - 1;
+    long long t = atom_add_acq_rel(&ctl->rank_blocks[rank], 1u);
+    atom_add_acq_rel(&ctl->arrived, 1u);
+    unsigned spins = 0;
+    while (ld_acquire(&ctl->arrived) < gridDim.x) {
+        if (++spins > limit) {
+            raise_status(status, QP_ERR_TIMEOUT);
+            return 1ll << 62;
+        }
+        __nanosleep(32);
+    }
+    for (unsigned q = 0; q < rank; ++q) t += __ldcg(&ctl->rank_blocks[q]);
+    return t;
+}
+
 // Decoupled look-back over a chain of tiles.  A tile first publishes its
 // aggregate (the number of particles it appends); the exclusive prefix is
 // then computed by one full warp with a 32-tile window: lane l inspects tile
@@ -1875,7 +1906,7 @@ __device__ __noinline__ void long_tile_loop(const StepArgs &a, const Problem *ta
 }
 
 // One launch = one step of every active problem.  Persistent blocks take
-// tiles by ticket (block b's first tile is b in a cooperative launch, every
+// tiles by ticket (a block's first tile is fixed in a cooperative launch, every
 // other ticket comes from an atomic counter, fetched while the tile before it
 // runs); tickets enumerate, problem after problem, its electron tiles,
 // positron tiles and photon tiles, so within each problem's chains start
@@ -1910,16 +1941,17 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // Tickets.  A tile must belong to a running block (its successors' look-
-    // backs wait on it).  A single problem on the mixed path is launched
-    // cooperatively (launch_step): every block is resident for the whole
-    // launch, so block b takes tile b at entry and later tickets come from
-    // the counter, offset by the grid; no block queues on the contended
-    // counter before its first tile.  The FP64 path and batches take every
-    // ticket from the counter, so a tile belongs to a block only once that
-    // block runs (a batch's launches are captured in graphs next to other
-    // streams' kernels; the FP64 path's one-launch-a-step runs of small
-    // problems, 4096 e- on 608 blocks, took 75 -> 108 us a step when
-    // launched cooperatively); the first atomic overlaps the reads of the
+    // backs wait on it).  A single problem on the mixed path, or of several
+    // steps a launch, is launched cooperatively (launch_step): every block is
+    // resident for the whole launch, so each has a fixed first tile (its own
+    // number, or spread_ticket's in launches of several steps) and later
+    // tickets come from the counter, offset by the grid; no block queues on
+    // the contended counter before its first tile.  An FP64 launch of one step
+    // and batches take every ticket from the counter, so a tile belongs to a
+    // block only once that block runs (a batch's launches are captured in
+    // graphs next to other streams' kernels; the FP64 path's one-launch-a-step
+    // runs of small problems, 4096 e- on 608 blocks, took 75 -> 108 us a step
+    // when launched cooperatively); the first atomic overlaps the reads of the
     // live counts below.  A block whose ticket is past the last tile leaves
     // without work.
     const int n_steps = BATCH ? 1 : single_steps(a.launch);
@@ -1940,13 +1972,18 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
         stage_pair_table<PREC, FK, R>(a, sm, &sh.bar[1]);
     }
 
+    const bool spread = !BATCH && n_steps > 1;
+    long long first_ticket = blockIdx.x;
+    if (spread && tid == 0)
+        first_ticket = spread_ticket(a.ctl, a.spin_limit, a.status);
+
     bool lep_loaded = false, ph_loaded = false;
     // a launch of several steps (all of its blocks are resident) takes them
     // one after the other, the blocks meeting at the end of each
 #pragma unroll 1
     for (int step = 0;; ++step) {
     if (tid == 0) {
-        sh.ticket[0] = fixed_first ? blockIdx.x : atomicAdd(&a.ctl->ticket, 1u);
+        sh.ticket[0] = fixed_first ? first_ticket : atomicAdd(&a.ctl->ticket, 1u);
         sh.tdone = 1u;
         sh.tclaim = sh.claim = 0u;
     }
@@ -2164,6 +2201,11 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
             }
         }
         __syncthreads();
+        if (spread && step == n_steps - 1) {
+            for (int k = tid; k < kSpreadSms; k += kTile) a.ctl->sm_blocks[k] = 0u;
+            if (tid < kSpreadRanks) a.ctl->rank_blocks[tid] = 0u;
+            if (tid == 0) a.ctl->arrived = 0u;
+        }
         // the next launch reads these after this one has ended, the next step
         // of this one once it has acquired the epoch
         if (tid == 0) {
