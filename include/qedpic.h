@@ -220,8 +220,10 @@ typedef struct {
  * slot (then emission index); photons emitted by electrons precede those of
  * positrons.  Particles that do not fit are counted as dropped and their
  * energy recorded; the step still completes.  The first step with species
- * larger than any stepped before grows the context's look-back scratch (one
- * allocation, synchronous); otherwise no allocation, no host synchronisation,
+ * larger than any stepped before grows the context's look-back scratch, and
+ * the first of a path, or of capacities that fill every warp several times
+ * over, its append scratch (74 MB, then up to 444 MB): an allocation each,
+ * synchronous; otherwise no allocation, no host synchronisation,
  * no host reads: the call can then be captured in a CUDA graph.  Up to eight
  * steps (one while launches are timed, see qp_profile_enable) are one launch
  * of the step kernel over every resident block of the GPU; on the mixed path,
