@@ -2201,7 +2201,8 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
             }
         }
         __syncthreads();
-        if (spread && step == n_steps - 1) {
+        // every block has its first ticket: it has counted this step
+        if (spread && step == 0) {
             for (int k = tid; k < kSpreadSms; k += kTile) a.ctl->sm_blocks[k] = 0u;
             if (tid < kSpreadRanks) a.ctl->rank_blocks[tid] = 0u;
             if (tid == 0) a.ctl->arrived = 0u;
