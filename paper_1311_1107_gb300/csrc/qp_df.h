@@ -234,13 +234,14 @@ QP_HD float hi_d(double d)
 }
 
 // Exact conversion of a float to double by integer instructions (normal
-// floats; zero and denormals give 0).
+// floats, infinities and NaN; zero and denormals give 0).
 QP_HD double f_to_d(float f)
 {
     const uint32_t b = f2u(f);
     const uint32_t e = (b >> 23) & 0xFFu;
     if (e == 0u) return 0.0;
-    return u2d(((uint64_t)(b & 0x80000000u) << 32) | ((uint64_t)(e + 896u) << 52) |
+    const uint32_t bias = e == 0xFFu ? 2u * 896u : 896u;
+    return u2d(((uint64_t)(b & 0x80000000u) << 32) | ((uint64_t)(e + bias) << 52) |
                ((uint64_t)(b & 0x7FFFFFu) << 29));
 }
 
