@@ -386,14 +386,16 @@ __device__ __forceinline__ R yee_interp(const float *__restrict__ F, const YeeSt
 }
 
 // A node's value in the gather's type; to FP64 by integer instructions (the
-// conversion unit is the FP64 pipe).
+// conversion unit is the FP64 pipe), denormals aside.
 template <typename R>
 __device__ __forceinline__ R node_value(float v)
 {
-    if constexpr (sizeof(R) == 8)
+    if constexpr (sizeof(R) == 8) {
+        if ((__float_as_uint(v) << 1) - 1u < 0xFFFFFFu) return (double)v;  // denormal
         return f_to_d(v);
-    else
+    } else {
         return v;
+    }
 }
 
 template <typename R>
