@@ -94,6 +94,20 @@ __device__ __forceinline__ double sqrt_rn(double x)
     return x > 0.0 ? root_of(x, rsqrt64(x)) : sqrt(x);
 }
 
+// 1/x rounded to nearest: the same correction of rcp64's reciprocal, exact but
+// for a mantissa of ones.  group_key's bins depend on its last bit: one unit
+// more or less moves a photon on the edge of two direction bins to the other,
+// and a product |u| r above 1 out of the first.  (Both checked on the host for
+// FP32 seeds within 2 units: 6e7 reciprocals, and 2e7 roots with the 14000
+// nearest to a tie.)
+__device__ __forceinline__ double rcp_rn(double x)
+{
+    const unsigned long long mantissa = (unsigned long long)__double_as_longlong(x) << 12;
+    if (!in_fp32_range(x) || mantissa == ~0ull << 12) return rcp64_ieee(x);
+    const double r = rcp64(x);
+    return fma(fma(-x, r, 1.0), r, r);
+}
+
 // The cell of one axis: the offset times the reciprocal of the cell size
 // (formed on the host), rounded down by the conversion; false outside the box
 // (NaN converts to the lowest integer).
@@ -128,7 +142,7 @@ __device__ unsigned long long group_key(const CoParams &C, double x, double y, d
     const double d = z_dom ? uz : y_dom ? uy : ux;
     const double p = z_dom ? ux : y_dom ? uz : uy, q = z_dom ? uy : y_dom ? ux : uz;
     const int face = 2 * (z_dom ? 2 : y_dom ? 1 : 0) + (__double2hiint(d) < 0 ? 1 : 0);
-    const double r = rcp64(fabs(d));
+    const double r = rcp_rn(fabs(d));  // p r and q r are in [-1, 1]
     const long long D = C.D;
     const long long ia = min((long long)__double2int_rd((p * r + 1.0) * C.half_D), D - 1);
     const long long ib = min((long long)__double2int_rd((q * r + 1.0) * C.half_D), D - 1);
