@@ -472,7 +472,9 @@ int qp_fill_yee2d(qp_ctx *ctx, const qp_pulse2d *p, const qp_field *grid, double
 /* s->n_steps cycles as above on the grid s->field with time step s->dt; jx,
  * jy, jz: device float arrays of ny rows of nx values on E's staggering, left
  * with the last cycle's current.  Five launches a cycle: J is zeroed by the
- * first B half step, both lepton species are deposited together. */
+ * first B half step, both lepton species are deposited together.  What
+ * qp_step rejects, and a missing current array, is rejected before anything is
+ * enqueued. */
 int qp_pic_step(qp_ctx *ctx, const qp_step_params *s, float *jx, float *jy, float *jz,
                 void *stream);
 

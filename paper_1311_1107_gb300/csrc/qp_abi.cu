@@ -709,18 +709,13 @@ void chain_words_of(const qp_ctx *ctx, const qp_step_params *s, size_t &lep, siz
     pho = tiles_of(cap(s->photon)) + 4;
 }
 
-}  // namespace
-
-int qp_step(qp_ctx *ctx, const qp_step_params *s, void *stream)
+// The launch of `s`: every check of it, the scratch it needs (grown here) and
+// the kernel's arguments but the first step and the number of steps.  Nothing
+// is enqueued.
+int prepare_step(qp_ctx *ctx, const qp_step_params *s, qp::StepArgs &a, int &grid, bool &long_ok)
 {
-    if (!ctx) return QP_ERR_NOT_INITIALIZED;
-    if (!s) return QP_ERR_INVALID_ARG;
-    qp::StepArgs a{};
     int st = build_problem(ctx, s, a.single);
-    if (st != QP_OK) return st;
-    if (s->n_steps == 0) return QP_OK;
-    DeviceGuard g(ctx->device);
-    if (!g.ok) return QP_ERR_CUDA;
+    if (st != QP_OK || s->n_steps == 0) return st;
     size_t lep = 0, pho = 0;
     chain_words_of(ctx, s, lep, pho);
     st = ensure_chain(ctx, lep > pho ? lep : pho);
@@ -742,9 +737,8 @@ int qp_step(qp_ctx *ctx, const qp_step_params *s, void *stream)
     for (int k = 0; k < 3; ++k)
         if (hs[k] != -1) cap_tiles += (int64_t)tiles_of(ctx->species[hs[k]].d.capacity);
     const int64_t resident = (int64_t)bpsm * ctx->num_sms;
-    const int grid = (int)(cap_tiles < resident ? (cap_tiles > 0 ? cap_tiles : 1) : resident);
-    const bool long_ok = qp::has_long_tiles(s->field.kind) &&
-                         qp::long_tiles(cap_tiles * qp::kWarps, grid);
+    grid = (int)(cap_tiles < resident ? (cap_tiles > 0 ? cap_tiles : 1) : resident);
+    long_ok = qp::has_long_tiles(s->field.kind) && qp::long_tiles(cap_tiles * qp::kWarps, grid);
     // For the resident blocks, whatever the grid, so that it grows a few times
     // at most: with the precision and when long tiles are first met.  A stash
     // that was outgrown stays until the context goes: a captured step may hold it.
@@ -759,16 +753,38 @@ int qp_step(qp_ctx *ctx, const qp_step_params *s, void *stream)
         ctx->stash_bytes = stash;
     }
     a.stash = ctx->d_stash;
-    cudaStream_t cs = (cudaStream_t)stream;
+    return QP_OK;
+}
+
+// Steps `first` .. `first + steps - 1` of a prepared launch.
+cudaError_t launch_steps(qp_ctx *ctx, const qp_step_params *s, qp::StepArgs &a, int grid,
+                         bool long_ok, int64_t first, int steps, cudaStream_t cs)
+{
+    a.single.step = (uint64_t)first;
+    a.launch = qp::single_launch(steps, long_ok);
+    return timed(ctx, 0, cs,
+                 [&] { return qp::launch_step(a, s->precision, s->field.kind, false, grid, cs); });
+}
+
+}  // namespace
+
+int qp_step(qp_ctx *ctx, const qp_step_params *s, void *stream)
+{
+    if (!ctx) return QP_ERR_NOT_INITIALIZED;
+    if (!s) return QP_ERR_INVALID_ARG;
+    DeviceGuard g(ctx->device);
+    if (!g.ok) return QP_ERR_CUDA;
+    qp::StepArgs a{};
+    int grid = 1;
+    bool long_ok = false;
+    const int st = prepare_step(ctx, s, a, grid, long_ok);
+    if (st != QP_OK) return st;
     // several steps a launch; one each while launches are timed
     const int per = ctx->profiling ? 1 : qp::kStepsPerLaunch;
     for (int32_t k = 0; k < s->n_steps; k += per) {
         const int steps = s->n_steps - k < per ? s->n_steps - k : per;
-        P.step = (uint64_t)(s->step + k);
-        a.launch = qp::single_launch(steps, long_ok);
-        cudaError_t e = timed(ctx, 0, cs, [&] {
-            return qp::launch_step(a, s->precision, s->field.kind, false, grid, cs);
-        });
+        cudaError_t e = launch_steps(ctx, s, a, grid, long_ok, s->step + k, steps,
+                                     (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_status(e);
     }
     return QP_OK;
@@ -1211,22 +1227,21 @@ int qp_pic_step(qp_ctx *ctx, const qp_step_params *s, float *jx, float *jy, floa
     }
     DeviceGuard d(ctx->device);
     if (!d.ok) return QP_ERR_CUDA;
+    // every check and allocation of the steps before the grid is touched
+    qp::StepArgs a{};
+    int blocks = 1;
+    bool long_ok = false;
+    const int st = prepare_step(ctx, s, a, blocks, long_ok);
+    if (st != QP_OK) return st;
     cudaStream_t cs = (cudaStream_t)stream;
     float *const j[3] = {jx, jy, jz};
-    qp_step_params one = *s;
-    one.n_steps = 1;
     for (int32_t k = 0; k < s->n_steps; ++k) {
-        one.step = s->step + k;
         cudaError_t e = qp::launch_yee_b(g, 0.5 * s->dt, j, ctx->num_sms, cs);
-        if (e != cudaSuccess) return cuda_status(e);
-        const int st = qp_step(ctx, &one, stream);
-        if (st != QP_OK) return st;
-        if (n_lep) {
+        if (e == cudaSuccess) e = launch_steps(ctx, s, a, blocks, long_ok, s->step + k, 1, cs);
+        if (e == cudaSuccess && n_lep)
             e = qp::launch_deposit(lep[0], q[0], lep[1], q[1], s->dt, g, jx, jy, jz,
                                    ctx->d_status, ctx->num_sms, cs);
-            if (e != cudaSuccess) return cuda_status(e);
-        }
-        e = qp::launch_yee_b(g, 0.5 * s->dt, nullptr, ctx->num_sms, cs);
+        if (e == cudaSuccess) e = qp::launch_yee_b(g, 0.5 * s->dt, nullptr, ctx->num_sms, cs);
         if (e == cudaSuccess) e = qp::launch_yee_e(g, jx, jy, jz, s->dt, ctx->num_sms, cs);
         if (e != cudaSuccess) return cuda_status(e);
     }
