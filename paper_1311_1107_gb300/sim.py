@@ -205,12 +205,16 @@ class Simulation:
 
     def run(self, n_steps: int, stream=None) -> int:
         if self.pic_pulse is not None:
-            # PIC cycles (E^n and B^(n-1/2) stored between cycles)
-            self.params.step = self.step_index
-            self.params.n_steps = int(n_steps)
+            # PIC cycles (E^n and B^(n-1/2) stored between cycles), a call each:
+            # after an error the index is that of the cycles the grid has taken
             j = [self.J[k].data_ptr() for k in range(3)]
-            st = Q.qp_pic_step(self.ctx, self.params, j[0], j[1], j[2], stream_handle(stream))
-            self.step_index += int(n_steps)
+            sh = stream_handle(stream)
+            self.params.n_steps = 1
+            st = 0
+            for _ in range(int(n_steps)):
+                self.params.step = self.step_index
+                st = max(st, Q.qp_pic_step(self.ctx, self.params, j[0], j[1], j[2], sh))
+                self.step_index += 1
             return st
         if self.pulse is not None:
             # fields refilled from the pulse at each step's time, then the step
