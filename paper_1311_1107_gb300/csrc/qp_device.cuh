@@ -314,7 +314,7 @@ static __device__ __noinline__ double rcp64_ieee(double x) { return 1.0 / x; }
 __device__ __forceinline__ double rcp64(double x)
 {
     if (!in_fp32_range(x)) return rcp64_ieee(x);
-    const double y = f_to_d(__fdividef(1.0f, hi_d(x)));
+    const double y = finite_to_d(__fdividef(1.0f, hi_d(x)));
     const double e = fma(-x, y, 1.0);
     return fma(y, fma(e, e, e), y);
 }
@@ -325,7 +325,7 @@ static __device__ __noinline__ double rsqrt64_ieee(double x) { return 1.0 / sqrt
 __device__ __forceinline__ double rsqrt64(double x)
 {
     if (!in_fp32_range(x)) return rsqrt64_ieee(x);
-    const double y = f_to_d(rsqrtf(hi_d(x)));
+    const double y = finite_to_d(rsqrtf(hi_d(x)));
     const double e = fma(-(x * y), y, 1.0);
     return fma(y * e, fma(e, 0.375, 0.5), y);
 }
@@ -386,13 +386,15 @@ __device__ __forceinline__ R yee_interp(const float *__restrict__ F, const YeeSt
 }
 
 // A node's value in the gather's type; to FP64 by integer instructions (the
-// conversion unit is the FP64 pipe), denormals aside.
+// conversion unit is the FP64 pipe) unless it is denormal, infinite or NaN.
 template <typename R>
 __device__ __forceinline__ R node_value(float v)
 {
     if constexpr (sizeof(R) == 8) {
-        if ((__float_as_uint(v) << 1) - 1u < 0xFFFFFFu) return (double)v;  // denormal
-        return f_to_d(v);
+        // exponents 255 and 0 become the lowest two; 0x01000000 is a zero
+        const unsigned u = (__float_as_uint(v) << 1) + 0x01000000u;
+        if (u < 0x02000000u && u != 0x01000000u) return (double)v;
+        return finite_to_d(v);
     } else {
         return v;
     }

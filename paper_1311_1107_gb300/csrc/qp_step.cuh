@@ -270,7 +270,7 @@ __device__ __forceinline__ double photon_depth(const Problem &P, const StepTime 
     if constexpr (PREC == kFP64)
         return -log(u53(r.x, r.y));
     else
-        return f_to_d(-logf(u53f(r.x, r.y)));
+        return finite_to_d(-logf(u53f(r.x, r.y)));
 }
 
 // Entries of a warp's queue of emitters: long parts, fewer than 32 wait while
@@ -524,7 +524,7 @@ __device__ __forceinline__ bool lepton_push(const StepArgs &a, const Problem &P,
         sink.tables();  // tables are needed from here on
         const float chi = chi_mixed_auto(uxd, uyd, uzd, dux, duy, duz, ux, uy, uz, gam, E, B,
                                          m.inv_aS, m.inv_aS_lo);
-        sink.chi(f_to_d(chi));
+        sink.chi(finite_to_d(chi));
         float dvx = 0.0f, dvy = 0.0f, dvz = 0.0f;
         float dtau = 0.0f;
 
@@ -696,11 +696,11 @@ __device__ __forceinline__ void lepton_events(const StepArgs &a, const Problem &
                 // the photons' direction goes to the append record now
                 // (fewer values live through the loop)
                 const float ip = pmag > 0.0f ? 1.0f / pmag : 0.0f;
-                sink.direction(f_to_d(ux * ip), f_to_d(uy * ip), f_to_d(uz * ip));
+                sink.direction(finite_to_d(ux * ip), finite_to_d(uy * ip), finite_to_d(uz * ip));
             }
             ++n_emit;
             if (gg > m.gmin) {
-                sink.photon(nph, f_to_d(gg), k);
+                sink.photon(nph, finite_to_d(gg), k);
                 ++nph;
             } else {
                 ++n_sub;
@@ -742,7 +742,7 @@ __device__ __forceinline__ void lepton_events(const StepArgs &a, const Problem &
         sink.template put<4>(add_fd(s.uy, duy));
         if (duz != 0.0f) sink.template put<5>(add_fd(s.uz, duz));
         sink.template put<6>(merge_df(TAU));
-        if (n_sub) o.e_sub = f_to_d(esub_f);
+        if (n_sub) o.e_sub = finite_to_d(esub_f);
     }
     o.n_emit = n_emit;
     o.nph = nph;
@@ -1109,11 +1109,11 @@ __device__ __forceinline__ bool photon_step(const StepArgs &a, const Problem &P,
                 s2 > 0.0f ? over_aS(g * sqrtf(s2), m.inv_aS, m.inv_aS_lo) : 0.0f;
             const float Tr = rate32<2>(T, chi, clamped);
             const float dtau = m.C_rate * Tr / g * m.dt;
-            if (Ph.chi) Ph.chi[i] = f_to_d(chi);
+            if (Ph.chi) Ph.chi[i] = finite_to_d(chi);
             const df2 TAU = split_d(taud);
             if (dtau > 0.0f && !(TAU.hi > dtau || (TAU.hi == dtau && TAU.lo > 0.0f))) {
                 decayed = true;
-                chi_d = f_to_d(chi);
+                chi_d = finite_to_d(chi);
                 Ph.tau[i] = -1.0;
             } else if (dtau != 0.0f) {
                 Ph.tau[i] = add_fd(taud, -dtau);
@@ -1169,10 +1169,10 @@ __device__ __forceinline__ void write_pairs(const StepArgs &a, const Problem &P,
                     a.tab.Cp2, a.tab.Qp2, a.tab.Gp, a.tab.Ep, hi_d(chi), u53_pair(r1.x, r1.y),
                     u53_pair_complement(r1.x, r1.y), (float)(kSpSpan / (kNNode - 1)), false,
                     clamped);
-                v = f_to_d(vf.x);
-                om = f_to_d(vf.omx);
-                tm = f_to_d(-logf(u53f(r1.z, r1.w)));
-                tp = f_to_d(-logf(u53f(r2.x, r2.y)));
+                v = finite_to_d(vf.x);
+                om = finite_to_d(vf.omx);
+                tm = finite_to_d(-logf(u53f(r1.z, r1.w)));
+                tp = finite_to_d(-logf(u53f(r2.x, r2.y)));
             }
             const int64_t se = be + ord, spo = bp + ord;
             El.x[se] = px;
