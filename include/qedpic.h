@@ -631,6 +631,16 @@ int qp_profile_read(qp_ctx *ctx, double ms[3], int64_t launches[3]);
  */
 int qp_selftest_wait_timeout(qp_ctx *ctx, uint32_t spin_limit);
 
+/*
+ * The same for the waits between the steps of one launch: launches of which
+ * one block comes late, so that the other blocks' waits for it run out (about
+ * spin_limit sleeps of 64 ns), then one without.  Returns QP_ERR_TIMEOUT when
+ * the first ones raised it, the last one raised nothing, and each left the
+ * context's control words as it found them; QP_ERR_CUDA otherwise.  Clears the
+ * sticky status.  Synchronous; no step of the context may be in flight.
+ */
+int qp_selftest_step_timeout(qp_ctx *ctx, uint32_t spin_limit);
+
 /* Static, NUL-terminated name of a status code. */
 const char *qp_status_string(int status);
 

@@ -1421,3 +1421,37 @@ int qp_selftest_wait_timeout(qp_ctx *ctx, uint32_t spin_limit)
 }
 
 }  // extern "C"
+int qp_selftest_step_timeout(qp_ctx *ctx, uint32_t spin_limit)
+{
+    if (!ctx) return QP_ERR_NOT_INITIALIZED;
+    DeviceGuard g(ctx->device);
+    if (!g.ok) return QP_ERR_CUDA;
+    // the first step's end, then the blocks' start, run out; then nothing does
+    const int late[3] = {1, 2, 0};
+    int status[3] = {0, 0, 0};
+    bool clean = true;
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
+        qp::StepCtl before, after;
+        e = cudaMemset(ctx->d_status, 0, sizeof(int));
+        if (e == cudaSuccess)
+            e = cudaMemcpy(&before, ctx->d_ctl, sizeof(before), cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess)
+            e = qp::launch_step_end_selftest(ctx->d_ctl, late[k], late[k] ? spin_limit : kSpinLimit,
+                                             ctx->d_status, 0);
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        if (e == cudaSuccess)
+            e = cudaMemcpy(&after, ctx->d_ctl, sizeof(after), cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess)
+            e = cudaMemcpy(&status[k], ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost);
+        // a new epoch, and nothing else changed
+        clean = clean && after.epoch != before.epoch;
+        after.epoch = before.epoch;
+        clean = clean && memcmp(&after, &before, sizeof(after)) == 0;
+    }
+    if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, sizeof(int));
+    if (e != cudaSuccess) return cuda_status(e);
+    if (!clean || status[2] != 0) return QP_ERR_CUDA;
+    return status[0] == status[1] ? status[0] : QP_ERR_CUDA;
+}
+

@@ -92,16 +92,21 @@ struct StepTime {
 };
 
 // Device-resident control block of a launch sequence: the tile ticket, the
-// count of finished blocks and the launch epoch that tags look-back words.  Blocks count their end in
-// kDoneGroups group counters (one 32-byte sector each) and the last of each
-// group in `done`: no counter sees more than a few tens of atomics at once.
+// epoch that tags look-back words (it advances with every step), whether the
+// launch has been given up (see abandon_launch), and the counts of blocks that
+// have ended a step.  Blocks count in kDoneGroups group counters (one 32-byte
+// sector each) and the last of each group in `done`: no counter sees more than
+// a few tens of atomics at once.  Row 1 counts the end of a launch's last step,
+// where every block comes by, row 0 the ends of the steps before it.  Between
+// launches everything but the epoch is 0.
 constexpr int kDoneGroups = 32;
 // The spread of a launch's first tiles (spread_ticket): blocks met on each SM
 // (SM ids modulo kSpreadSms) and as each SM's n-th, and blocks counted.
 constexpr int kSpreadSms = 256, kSpreadRanks = 32;
 struct StepCtl {
-    unsigned ticket, done, epoch, arrived;
-    unsigned grp[kDoneGroups][8];
+    unsigned ticket, epoch, abandoned, arrived;
+    unsigned done[2];
+    unsigned grp[2][kDoneGroups][8];
     unsigned sm_blocks[kSpreadSms], rank_blocks[kSpreadRanks];
 };
 

@@ -29,6 +29,35 @@ cudaError_t launch_wait_selftest(unsigned long long *words, unsigned spin_limit,
     return cudaGetLastError();
 }
 
+// The ends of a launch of three steps, one thread a block.  late 1: block 0 comes
+// to the end of the first step only after another block's wait for it ran out;
+// late 2: it counts as started only then.  Every other wait of a block is for
+// blocks that do not wait for it (bounded all the same).
+__global__ void k_step_end_selftest(StepCtl *ctl, int late, unsigned spin_limit, int *status)
+{
+    constexpr int kSteps = 3;
+    const bool is_late = late && blockIdx.x == 0;
+    unsigned epoch = __ldcg(&ctl->epoch);
+    if (is_late)
+        for (unsigned k = 0; k < (1u << 22) && !*(volatile unsigned *)&ctl->abandoned; ++k)
+            __nanosleep(256);
+    if (late == 2) (void)spread_ticket(ctl, spin_limit, status);
+    for (int step = 0;; ++step) {
+        if (last_block(ctl, step, kSteps)) end_step(ctl, epoch, step + 1 == kSteps);
+        if (step + 1 == kSteps || !next_step(ctl, epoch, spin_limit, status)) return;
+        ++epoch;
+    }
+}
+
+// More blocks than groups of counters; all resident (a cooperative launch).
+cudaError_t launch_step_end_selftest(StepCtl *ctl, int late, unsigned spin_limit, int *status,
+                                     cudaStream_t st)
+{
+    void *args[] = {(void *)&ctl, (void *)&late, (void *)&spin_limit, (void *)&status};
+    return cudaLaunchCooperativeKernel((const void *)k_step_end_selftest, dim3(2 * kDoneGroups + 3),
+                                       dim3(1), args, 0, st);
+}
+
 // -------------------------------------------------------------------- initial optical depth
 
 __global__ void k_init_tau(double *tau, int64_t first, int64_t count, int64_t id_base,

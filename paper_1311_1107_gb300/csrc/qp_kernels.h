@@ -68,6 +68,8 @@ struct DiagOut {
 cudaError_t launch_diag(const SpeciesDev &S, int is_photon, const DiagOut &o, cudaStream_t st);
 cudaError_t launch_wait_selftest(unsigned long long *words, unsigned spin_limit, int *status,
                                  cudaStream_t st);
+cudaError_t launch_step_end_selftest(StepCtl *ctl, int late, unsigned spin_limit, int *status,
+                                     cudaStream_t st);
 
 // A 2D Yee grid (qp_pic.cu): six float components, ny rows of nx values.
 struct YeeGrid {

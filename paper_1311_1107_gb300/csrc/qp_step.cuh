@@ -77,20 +77,104 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
     return v;
 }
 
+// The control block as a launch finds it, its epoch past every tag that a step
+// of this launch has used; one thread, once every block has counted its end.
+__device__ __noinline__ void clear_ctl(StepCtl *ctl)
+{
+    const unsigned epoch = *(volatile unsigned *)&ctl->epoch;
+    unsigned *const w = reinterpret_cast<unsigned *>(ctl);
+#pragma unroll 1
+    for (int k = 0; k < (int)(sizeof(StepCtl) / sizeof(unsigned)); ++k)
+        *(volatile unsigned *)(w + k) = w + k == &ctl->epoch ? epoch + 1u : 0u;
+}
+
+// One thread counts its block's end of a step (of a launch's last step: fin);
+// true in the last block.  The counts are acquire-release atomics: a count
+// releases the block's writes (every thread's: the barrier that closed its last
+// flush orders them before this thread's count) and the group's last count
+// acquires the group's, so the last block sees every block's pending counts.
+__device__ __forceinline__ bool count_block(StepCtl *ctl, bool fin)
+{
+    const unsigned g = blockIdx.x % kDoneGroups;
+    const unsigned in_group = (gridDim.x - 1 - g) / kDoneGroups + 1;
+    const unsigned groups = gridDim.x < kDoneGroups ? gridDim.x : kDoneGroups;
+    bool last = false;
+    if (atom_add_acq_rel(&ctl->grp[fin][g][0], 1u) == in_group - 1) {
+        ctl->grp[fin][g][0] = 0u;  // every block of the group has counted
+        last = atom_add_acq_rel(&ctl->done[fin], 1u) == groups - 1;
+    }
+    return last;
+}
+
+// The last block of a launch of several steps finds whether it was abandoned
+// (one thread): it then has no whole step to publish, and leaves the control
+// block clean, as no block has anything left to count: each has ended the
+// launch's last step or abandoned.
+__device__ __forceinline__ bool was_abandoned(StepCtl *ctl)
+{
+    if (!*(volatile unsigned *)&ctl->abandoned) return false;
+    clear_ctl(ctl);
+    return true;
+}
+
+// One thread ends its block's step `step`: true in the last block, which
+// publishes the step.
+__device__ __noinline__ bool last_block(StepCtl *ctl, int step, int n_steps)
+{
+    const bool fin = step + 1 == n_steps;
+    bool last = count_block(ctl, fin);
+    if (last && n_steps > 1 && fin) last = !was_abandoned(ctl);
+    return last;
+}
+
+// A block whose wait for the others ran out leaves a launch of several steps;
+// one thread.  The others see it at their next wait and leave too (this
+// block's tiles are missing), and the last to come by, here or at the end of
+// the last step, clears the control block.
+__device__ __noinline__ void abandon_launch(StepCtl *ctl)
+{
+    atomicExch(&ctl->abandoned, 1u);
+    if (count_block(ctl, true)) clear_ctl(ctl);
+}
+
+// The last block's end of a step, one thread: the next launch reads the control
+// block after this one has ended, the next step of this one once it has
+// acquired the epoch.
+__device__ __forceinline__ void end_step(StepCtl *ctl, unsigned epoch, bool fin)
+{
+    *(volatile unsigned *)&ctl->ticket = 0u;
+    *(volatile unsigned *)&ctl->done[fin] = 0u;
+    if (!fin)
+        st_release(&ctl->epoch, epoch + 1u);
+    else
+        *(volatile unsigned *)&ctl->epoch = epoch + 1u;
+}
+
 // One thread waits until the launch's epoch has left `epoch` (bounded; false
-// and the status on a time-out).
-__device__ __noinline__ bool await_epoch(const unsigned *p, unsigned epoch, unsigned limit,
-                                         int *status)
+// and the status on a time-out, false when another block gave the launch up).
+__device__ __forceinline__ bool await_epoch(const StepCtl *ctl, unsigned epoch, unsigned limit,
+                                            int *status)
 {
     unsigned spins = 0;
-    while (ld_acquire(p) == epoch) {
-        if (++spins > limit) {
+    while (ld_acquire(&ctl->epoch) == epoch) {
+        if (++spins % 256u == 0u && *(const volatile unsigned *)&ctl->abandoned) return false;
+        if (spins > limit) {
             raise_status(status, QP_ERR_TIMEOUT);
             return false;
         }
         __nanosleep(64);
     }
     return true;
+}
+
+// One thread waits for the launch's next step; false if it was given up.  (This
+// and last_block are called: their values would take registers from the tile
+// loops, 4.2e6-slot steps 1 % longer.)
+__device__ __noinline__ bool next_step(StepCtl *ctl, unsigned epoch, unsigned limit, int *status)
+{
+    const bool go = await_epoch(ctl, epoch, limit, status);
+    if (!go) abandon_launch(ctl);
+    return go;
 }
 
 // The first ticket of a block of a cooperative launch of several steps: 0 ..
@@ -101,9 +185,9 @@ __device__ __noinline__ bool await_epoch(const unsigned *p, unsigned epoch, unsi
 //   FP64   4096 electrons 1124 / 761, 8000 1131 / 821, 20000 1135 / 970, a
 //          cascade of 16384 with diagnostics 1554 / 1441;
 //   mixed  4096 458 / 424, 8000 556 / 472, 20000 and 40000 photons 570 / 510.
-// One thread a block; every block is resident, so the wait for all of them ends
-// (it is bounded; no tile and the status on a time-out).  It costs some 2 us, so
-// a launch of one step does without.
+// One thread a block; every block is resident, so the wait for all of them ends.
+// It is bounded: a block whose wait runs out abandons the launch and takes no
+// tile in it.  It costs some 2 us, so a launch of one step does without.
 __device__ __noinline__ long long spread_ticket(StepCtl *ctl, unsigned limit, int *status)
 {
     unsigned sm;
@@ -116,6 +200,7 @@ __device__ __noinline__ long long spread_ticket(StepCtl *ctl, unsigned limit, in
     while (ld_acquire(&ctl->arrived) < gridDim.x) {
         if (++spins > limit) {
             raise_status(status, QP_ERR_TIMEOUT);
+            atomicExch(&ctl->abandoned, 1u);
             return 1ll << 62;
         }
         __nanosleep(32);
@@ -2046,7 +2131,7 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
             // a round without a tile empties the ring before the block leaves
             const bool drain = leave && q_lo != q;
             if (leave && !drain) {
-                if (BATCH || step == n_steps - 1)
+                if (BATCH || step + 1 == n_steps)
                     leave_problem(a, BATCH ? sh.prob : a.single, cur, bs);
                 if (!more) break;
                 if constexpr (BATCH) {
@@ -2157,22 +2242,8 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
         lep_loaded = ph_loaded = true;
     }
 
-    // ---- the last block to finish publishes the step of every problem:
-    // the last block of each group counts in `done`, the last of those is it
-    // The counts are acquire-release atomics: a count releases the block's
-    // writes (every thread's: the barrier that closed its last flush orders
-    // them before thread 0's count) and the group's last count acquires the
-    // group's, so the last block sees every block's pending counts.
-    if (tid == 0) {
-        const unsigned g = blockIdx.x % kDoneGroups;
-        const unsigned in_group = (gridDim.x - 1 - g) / kDoneGroups + 1;
-        const unsigned groups = gridDim.x < kDoneGroups ? gridDim.x : kDoneGroups;
-        sh.last = 0;
-        if (atom_add_acq_rel(&a.ctl->grp[g][0], 1u) == in_group - 1) {
-            a.ctl->grp[g][0] = 0u;  // every block of the group has counted
-            sh.last = atom_add_acq_rel(&a.ctl->done, 1u) == groups - 1;
-        }
-    }
+    // ---- the last block to finish publishes the step of every problem
+    if (tid == 0) sh.last = last_block(a.ctl, step, n_steps);
     __syncthreads();
     if (sh.last) {
         // thread 0 acquired with its count; the other threads' reads (a
@@ -2207,21 +2278,12 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
             if (tid < kSpreadRanks) a.ctl->rank_blocks[tid] = 0u;
             if (tid == 0) a.ctl->arrived = 0u;
         }
-        // the next launch reads these after this one has ended, the next step
-        // of this one once it has acquired the epoch
-        if (tid == 0) {
-            *((volatile unsigned *)&a.ctl->ticket) = 0u;
-            *((volatile unsigned *)&a.ctl->done) = 0u;
-            if (step < n_steps - 1)
-                st_release(&a.ctl->epoch, epoch + 1u);
-            else
-                *((volatile unsigned *)&a.ctl->epoch) = epoch + 1u;
-        }
+        if (tid == 0) end_step(a.ctl, epoch, step + 1 == n_steps);
     }
-    if (BATCH || step == n_steps - 1) break;
-    if (tid == 0) sh.go = await_epoch(&a.ctl->epoch, epoch, a.spin_limit, a.status);
+    if (BATCH || step + 1 == n_steps) break;
+    if (tid == 0) sh.go = next_step(a.ctl, epoch, a.spin_limit, a.status);
     __syncthreads();
-    if (!sh.go) break;  // timed out: the status says so
+    if (!sh.go) break;  // given up: the status says so
     ++epoch;
     }
     // the copies of the tables land before the block leaves

@@ -126,7 +126,7 @@ class qp_coalesce_stats(C.Structure):
 EXPORTS = ("qp_init_tables", "qp_destroy", "qp_create_species", "qp_init_optical_depth",
            "qp_species_copy", "qp_step_host",
            "qp_step", "qp_diagnostics", "qp_export_tables", "qp_reset_counters",
-           "qp_selftest_wait_timeout", "qp_profile_enable", "qp_profile_read",
+           "qp_selftest_wait_timeout", "qp_selftest_step_timeout", "qp_profile_enable", "qp_profile_read",
            "qp_diagnostics_noalloc", "qp_status_string", "qp_destroy_species",
            "qp_batch_create", "qp_batch_destroy", "qp_batch_scratch_words", "qp_batch_set",
            "qp_batch_clear", "qp_batch_step", "qp_batch_progress", "qp_coalesce_photons",
@@ -164,6 +164,7 @@ def lib(build_if_missing: bool = False):
         L.qp_export_tables.argtypes = [vp, C.POINTER(qp_tables_export)]
         L.qp_reset_counters.argtypes = [vp, i32]
         L.qp_selftest_wait_timeout.argtypes = [vp, C.c_uint32]
+        L.qp_selftest_step_timeout.argtypes = [vp, C.c_uint32]
         L.qp_profile_enable.argtypes = [vp, C.c_int]
         L.qp_profile_read.argtypes = [vp, C.POINTER(C.c_double), C.POINTER(C.c_int64)]
         L.qp_destroy_species.argtypes = [vp, i32]
@@ -281,6 +282,12 @@ def qp_reset_counters(ctx, handle: int) -> int:
 def qp_selftest_wait_timeout(ctx, spin_limit: int) -> int:
     """Status raised by a deliberately unsatisfiable, bounded device wait."""
     return lib().qp_selftest_wait_timeout(ctx, int(spin_limit))
+
+
+def qp_selftest_step_timeout(ctx, spin_limit: int) -> int:
+    """QP_ERR_TIMEOUT when launches whose blocks wait in vain for one another
+    raise it and leave the context as they found it."""
+    return lib().qp_selftest_step_timeout(ctx, int(spin_limit))
 
 
 def qp_profile_enable(ctx, enable: bool = True) -> int:
