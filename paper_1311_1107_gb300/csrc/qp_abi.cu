@@ -57,6 +57,9 @@ struct qp_ctx {
     unsigned long long *d_chain = nullptr;  // lepton chain then photon chain
     size_t chain_words = 0;           // words per chain
     double *d_diag = nullptr;         // partials of the diagnostics' blocks
+    // one qp_diagnostics at a time uses d_diag and these, from its launch until
+    // the host has read the copy
+    std::mutex diag_lock;
     qp::DiagRead *d_read = nullptr;   // what qp_diagnostics reads
     qp::DiagRead *h_read = nullptr;   // (pinned)
     double *d_stash = nullptr;        // append records of qp_step launches
@@ -1092,6 +1095,7 @@ int qp_step_fused(qp_ctx *ctx, const qp_step_params *s, int32_t fuse, void *stre
     for (int k = 0; k < 2; ++k) {
         const int64_t cap = hs[k] == -1 ? 0 : ctx->species[hs[k]].d.capacity;
         if (n[k] < 0 || n[k] > cap) return QP_ERR_INVALID_ARG;
+    std::lock_guard<std::mutex> lock(ctx->diag_lock);
     }
     const long long tiles_e = (n[0] + 31) / 32, tiles = tiles_e + (n[1] + 31) / 32;
     const int K = fuse < s->n_steps ? fuse : s->n_steps;
