@@ -712,10 +712,33 @@ void chain_words_of(const qp_ctx *ctx, const qp_step_params *s, size_t &lep, siz
     pho = tiles_of(cap(s->photon)) + 4;
 }
 
+// The context's append scratch holds `words` doubles from here on (an
+// allocation, synchronous, when it grows; none while `cs` is being captured).
+// One that was outgrown stays until the context goes: a captured step may hold it.
+int grow_stash(qp_ctx *ctx, size_t words, cudaStream_t cs)
+{
+    const size_t bytes = words * sizeof(double);
+    if (bytes <= ctx->stash_bytes) return QP_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(cs, &cap);
+    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return QP_ERR_CUDA;
+    double *p = nullptr;
+    if (e == cudaSuccess) e = cudaMalloc(&p, bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();  // reported here: not to the launch that may follow
+        return cuda_status(e);
+    }
+    if (ctx->d_stash) ctx->old_stash.push_back(ctx->d_stash);
+    ctx->d_stash = p;
+    ctx->stash_bytes = bytes;
+    return QP_OK;
+}
+
 // The launch of `s`: every check of it, the scratch it needs (grown here) and
 // the kernel's arguments but the first step and the number of steps.  Nothing
 // is enqueued.
-int prepare_step(qp_ctx *ctx, const qp_step_params *s, qp::StepArgs &a, int &grid, bool &long_ok)
+int prepare_step(qp_ctx *ctx, const qp_step_params *s, qp::StepArgs &a, int &grid, bool &long_ok,
+                 cudaStream_t cs)
 {
     int st = build_problem(ctx, s, a.single);
     if (st != QP_OK || s->n_steps == 0) return st;
@@ -741,19 +764,16 @@ int prepare_step(qp_ctx *ctx, const qp_step_params *s, qp::StepArgs &a, int &gri
         if (hs[k] != -1) cap_tiles += (int64_t)tiles_of(ctx->species[hs[k]].d.capacity);
     const int64_t resident = (int64_t)bpsm * ctx->num_sms;
     grid = (int)(cap_tiles < resident ? (cap_tiles > 0 ? cap_tiles : 1) : resident);
-    long_ok = qp::has_long_tiles(s->field.kind) && qp::long_tiles(cap_tiles * qp::kWarps, grid);
-    // For the resident blocks, whatever the grid, so that it grows a few times
-    // at most: with the precision and when long tiles are first met.  A stash
-    // that was outgrown stays until the context goes: a captured step may hold it.
-    const size_t stash = (size_t)resident * qp::stash_words(long_ok) * sizeof(double);
-    if (stash > ctx->stash_bytes) {
-        // grows (an allocation, synchronous)
-        double *p = nullptr;
-        cudaError_t e = cudaMalloc(&p, stash);
-        if (e != cudaSuccess) return cuda_status(e);
-        if (ctx->d_stash) ctx->old_stash.push_back(ctx->d_stash);
-        ctx->d_stash = p;
-        ctx->stash_bytes = stash;
+    // For the resident blocks, whatever the grid, so that the stash grows a few
+    // times at most: with the precision and when long tiles are first met.
+    // Where theirs cannot be had (during a capture, or short of memory) the
+    // steps keep to short tiles: the same results from a sixth of the room.
+    long_ok = qp::has_long_tiles(s->field.kind) &&
+              qp::long_tiles(cap_tiles * qp::kWarps, grid) &&
+              grow_stash(ctx, (size_t)resident * qp::stash_words(true), cs) == QP_OK;
+    if (!long_ok) {
+        st = grow_stash(ctx, (size_t)resident * qp::stash_words(false), cs);
+        if (st != QP_OK) return st;
     }
     a.stash = ctx->d_stash;
     return QP_OK;
@@ -780,7 +800,7 @@ int qp_step(qp_ctx *ctx, const qp_step_params *s, void *stream)
     qp::StepArgs a{};
     int grid = 1;
     bool long_ok = false;
-    const int st = prepare_step(ctx, s, a, grid, long_ok);
+    const int st = prepare_step(ctx, s, a, grid, long_ok, (cudaStream_t)stream);
     if (st != QP_OK) return st;
     // several steps a launch; one each while launches are timed
     const int per = ctx->profiling ? 1 : qp::kStepsPerLaunch;
@@ -1235,7 +1255,7 @@ int qp_pic_step(qp_ctx *ctx, const qp_step_params *s, float *jx, float *jy, floa
     qp::StepArgs a{};
     int blocks = 1;
     bool long_ok = false;
-    const int st = prepare_step(ctx, s, a, blocks, long_ok);
+    const int st = prepare_step(ctx, s, a, blocks, long_ok, (cudaStream_t)stream);
     if (st != QP_OK) return st;
     cudaStream_t cs = (cudaStream_t)stream;
     float *const j[3] = {jx, jy, jz};
