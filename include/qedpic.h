@@ -308,8 +308,9 @@ int qp_step_fused(qp_ctx *ctx, const qp_step_params *s, int32_t fuse, void *stre
  */
 typedef struct qp_batch qp_batch;
 
-/* Allocate a batch (device table, counters, pinned staging) for problems of
- * one precision (QP_FP64 / QP_MIXED) and field kind.  Synchronous.
+/* Allocate a batch (device table, counters, pinned staging, 42 to 74 MB of
+ * append scratch) for problems of one precision (QP_FP64 / QP_MIXED) and field
+ * kind.  Synchronous.
  * QP_ERR_INVALID_ARG unless 1 <= max_problems <= QP_MAX_BATCH. */
 int qp_batch_create(qp_ctx *ctx, int32_t max_problems, int32_t precision, int32_t field_kind,
                     qp_batch **out);
@@ -333,7 +334,10 @@ int qp_batch_scratch_words(qp_ctx *ctx, const qp_step_params *s, int64_t *words)
  * species' counters, copies the descriptor, and activates the slot last, so
  * the problem is stepped from the next launch on.  The host side returns
  * without waiting for the device (staging buffers are reused only after
- * their copy completed).  QP_ERR_INVALID_ARG for a bad slot, a precision or
+ * their copy completed).  The first time the slots set hold enough capacity for
+ * long tiles (4.4e6 slots on the mixed path, 2.5e6 in FP64) the batch allocates
+ * their append scratch (up to 444 MB); without the memory it keeps to short
+ * tiles, with the same results.  QP_ERR_INVALID_ARG for a bad slot, a precision or
  * field kind other than the batch's, too little scratch, or what qp_step
  * rejects.  The species' initial state (positions, momenta, optical depths,
  * live counts) must be in place, in stream order, before the next launch.

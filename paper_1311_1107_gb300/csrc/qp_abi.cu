@@ -823,7 +823,11 @@ struct qp_batch {
     long long *d_left = nullptr;      // [max] launches still to run (0 = idle slot)
     long long *d_pending = nullptr;   // [max][3]
     long long *d_work = nullptr;      // [max] live slots stepped so far
-    double *d_stash = nullptr;        // append records of the batch's launches
+    // append records of the batch's launches: short tiles', and long tiles' once
+    // the problems set call for them (launches in flight may hold the former)
+    double *d_stash = nullptr, *d_long_stash = nullptr;
+    qp::BatchStash *d_batch = nullptr, *h_batch = nullptr;  // device; pinned
+    std::vector<int64_t> subs;        // [max] sub-tiles of the slots' capacities
     qp::StepCtl *d_ctl = nullptr;
     // pinned staging of the descriptors copied by qp_batch_set; entry k is
     // reused only after the copy that read it has completed (its event)
@@ -847,6 +851,9 @@ void batch_release(qp_batch *b)
     cudaFree(b->d_pending);
     cudaFree(b->d_work);
     cudaFree(b->d_stash);
+    cudaFree(b->d_long_stash);
+    cudaFree(b->d_batch);
+    cudaFreeHost(b->h_batch);
     cudaFree(b->d_ctl);
     cudaFreeHost(b->h_stage);
     cudaFreeHost(b->h_stage_ctl);
@@ -889,9 +896,12 @@ int qp_batch_create(qp_ctx *ctx, int32_t max_problems, int32_t precision, int32_
     QP_TRY(cudaMemset(b->d_left, 0, n * sizeof(long long)));
     QP_TRY(cudaMalloc(&b->d_pending, 3 * n * sizeof(long long)));
     QP_TRY(cudaMemset(b->d_pending, 0, 3 * n * sizeof(long long)));
-    QP_TRY(cudaMalloc(&b->d_stash, (size_t)b->grid *
-                                       qp::stash_words(qp::has_long_tiles(field_kind)) *
-                                       sizeof(double)));
+    QP_TRY(cudaMalloc(&b->d_stash, (size_t)b->grid * qp::stash_words(false) * sizeof(double)));
+    QP_TRY(cudaMalloc(&b->d_batch, sizeof(qp::BatchStash)));
+    QP_TRY(cudaMallocHost(&b->h_batch, sizeof(qp::BatchStash)));
+    *b->h_batch = qp::BatchStash{b->d_stash, 0u, 0u};
+    QP_TRY(cudaMemcpy(b->d_batch, b->h_batch, sizeof(qp::BatchStash), cudaMemcpyHostToDevice));
+    b->subs.assign(n, 0);
     QP_TRY(cudaMalloc(&b->d_work, n * sizeof(long long)));
     QP_TRY(cudaMemset(b->d_work, 0, n * sizeof(long long)));
     QP_TRY(cudaMalloc(&b->d_ctl, sizeof(qp::StepCtl)));
@@ -942,6 +952,39 @@ int qp_batch_scratch_words(qp_ctx *ctx, const qp_step_params *s, int64_t *words)
     return QP_OK;
 }
 
+namespace {
+
+// Long tiles' append records once the slots set, `slot` with the problem `s`, can
+// hold enough particles for long tiles (in stream order; without the memory the
+// batch keeps to short tiles, with the same results).
+cudaError_t grow_batch_stash(qp_batch *b, int32_t slot, const qp_step_params *s, cudaStream_t cs)
+{
+    const int32_t hs[3] = {s->electron, s->positron, s->photon};
+    int64_t subs = 0, all = 0;
+    for (int k = 0; k < 3; ++k)
+        if (hs[k] != -1) subs += (b->ctx->species[hs[k]].d.capacity + 31) / 32;
+    b->subs[slot] = subs;
+    for (int64_t v : b->subs) all += v;
+    if (b->d_long_stash || !qp::has_long_tiles(b->field_kind) || !qp::long_tiles(all, b->grid))
+        return cudaSuccess;
+    // (another thread's capture of another stream does not mind)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return e;
+    e = cudaMalloc(&b->d_long_stash, (size_t)b->grid * qp::stash_words(true) * sizeof(double));
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+        b->d_long_stash = nullptr;
+        cudaGetLastError();
+        return cudaSuccess;
+    }
+    *b->h_batch = qp::BatchStash{b->d_long_stash, 1u, 0u};  // written once: nothing reads it yet
+    return cudaMemcpyAsync(b->d_batch, b->h_batch, sizeof(qp::BatchStash), cudaMemcpyHostToDevice,
+                           cs);
+}
+
+}  // namespace
+
 int qp_batch_set(qp_batch *b, int32_t slot, const qp_step_params *s, uint64_t *scratch,
                  int64_t scratch_words, void *stream)
 {
@@ -968,6 +1011,7 @@ int qp_batch_set(qp_batch *b, int32_t slot, const qp_step_params *s, uint64_t *s
     const int k = b->stage_next;
     b->stage_next = (k + 1) % (2 * b->max);
     cudaError_t e = cudaEventSynchronize(b->stage_ev[k]);  // the entry's last copy is done
+    if (e == cudaSuccess) e = grow_batch_stash(b, slot, s, cs);
     if (e != cudaSuccess) return cuda_status(e);
     b->h_stage[k] = P;
     b->h_stage_ctl[2 * k] = s->step;
@@ -997,6 +1041,7 @@ int qp_batch_clear(qp_batch *b, int32_t slot, void *stream)
     if (slot < 0 || slot >= b->max) return QP_ERR_INVALID_ARG;
     DeviceGuard g(b->ctx->device);
     if (!g.ok) return QP_ERR_CUDA;
+    b->subs[slot] = 0;
     return cuda_status(
         cudaMemsetAsync(b->d_left + slot, 0, sizeof(long long), (cudaStream_t)stream));
 }
@@ -1012,7 +1057,7 @@ int qp_batch_step(qp_batch *b, int32_t n_launches, void *stream)
     a.ctl = b->d_ctl;
     a.launch = b->max;
     a.problems = b->d_table;
-    a.stash = b->d_stash;
+    a.batch = b->d_batch;
     cudaStream_t cs = (cudaStream_t)stream;
     for (int32_t k = 0; k < n_launches; ++k) {
         cudaError_t e = timed(b->ctx, 0, cs, [&] {
@@ -1050,6 +1095,7 @@ int qp_diagnostics(qp_ctx *ctx, int32_t handle, qp_diag *out, void *stream)
     cudaStream_t st = (cudaStream_t)stream;
     const qp_species_desc &d = ctx->species[handle].d;
     qp::SpeciesDev S = species_dev(ctx, handle);
+    std::lock_guard<std::mutex> lock(ctx->diag_lock);
     const qp::DiagOut o{ctx->d_diag, ctx->d_read, ctx->d_stats + handle, ctx->d_status};
     cudaError_t e = qp::launch_diag(S, d.kind == QP_PHOTON, o, st);
     if (e == cudaSuccess)
@@ -1115,7 +1161,6 @@ int qp_step_fused(qp_ctx *ctx, const qp_step_params *s, int32_t fuse, void *stre
     for (int k = 0; k < 2; ++k) {
         const int64_t cap = hs[k] == -1 ? 0 : ctx->species[hs[k]].d.capacity;
         if (n[k] < 0 || n[k] > cap) return QP_ERR_INVALID_ARG;
-    std::lock_guard<std::mutex> lock(ctx->diag_lock);
     }
     const long long tiles_e = (n[0] + 31) / 32, tiles = tiles_e + (n[1] + 31) / 32;
     const int K = fuse < s->n_steps ? fuse : s->n_steps;
@@ -1444,7 +1489,6 @@ int qp_selftest_wait_timeout(qp_ctx *ctx, uint32_t spin_limit)
     return status;
 }
 
-}  // extern "C"
 int qp_selftest_step_timeout(qp_ctx *ctx, uint32_t spin_limit)
 {
     if (!ctx) return QP_ERR_NOT_INITIALIZED;
@@ -1479,3 +1523,4 @@ int qp_selftest_step_timeout(qp_ctx *ctx, uint32_t spin_limit)
     return status[0] == status[1] ? status[0] : QP_ERR_CUDA;
 }
 
+}  // extern "C"

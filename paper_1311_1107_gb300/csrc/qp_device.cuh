@@ -173,6 +173,13 @@ struct Problem {
     int32_t pad;
 };
 
+// The append records of a batch's launches, and whether they have room for long
+// tiles.  On the device: a captured launch takes what the batch has when it runs.
+struct BatchStash {
+    double *stash;
+    unsigned long_ok, pad;
+};
+
 struct StepArgs {
     TablesDev tab;
     StepCtl *ctl;
@@ -183,7 +190,10 @@ struct StepArgs {
     int32_t launch;                   // batch: problems in the table; single problem: see
                                       // single_launch
     const Problem *problems;          // a batch's device table
-    double *stash;                    // append records: stash_words() a block
+    union {
+        double *stash;                // append records: stash_words() a block
+        const BatchStash *batch;      // a batch's
+    };
     Problem single;
 };
 

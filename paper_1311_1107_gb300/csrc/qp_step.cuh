@@ -2040,12 +2040,13 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
     // live counts below.  A block whose ticket is past the last tile leaves
     // without work.
     const int n_steps = BATCH ? 1 : single_steps(a.launch);
-    const bool long_ok = has_long_tiles(FK) && (BATCH || single_long(a.launch));
+    const bool long_ok =
+        has_long_tiles(FK) && (BATCH ? __ldcg(&a.batch->long_ok) != 0u : single_long(a.launch));
     const bool fixed_first = !BATCH && (PREC != kFP64 || n_steps > 1);
     const unsigned tbase = fixed_first ? gridDim.x : 0u;
     const int np = BATCH ? a.launch : 1;
     const Problem *table = BATCH ? a.problems : &a.single;
-    double *const stash = a.stash + (size_t)blockIdx.x * stash_words(long_ok);
+    double *const stash = (BATCH ? a.batch->stash : a.stash) + (size_t)blockIdx.x * stash_words(long_ok);
     unsigned epoch = __ldcg(&a.ctl->epoch);
     clear_stats(bs);
     // the lepton tiles' rate tables, staged from the start by a thread of
