@@ -193,13 +193,14 @@ __device__ __forceinline__ float2 ldg2(const float2 *p) { return __ldg(p); }
 // The interval is the last node below the key: the guide entry, then a
 // forward scan of mostly none to two nodes.  An emission round is a chain of
 // dependent loads that nothing hides when a problem fills the GPU once, so
-// the entry's next four nodes are loaded together (RowWindow, both rows of a
+// the entry's next nodes are loaded together (RowWindow, both rows of a
 // sample before either is used): two round trips a sample, where a node at a
 // time of one row after the other took about ten (2D foil: 90 % of the warps
 // through their first tile's events after 24 us of a step).
+template <int NODES>
 struct RowWindow {
-    float2 edge;   // C_0 of the lower half, Q_last of the upper
-    float2 w[4];   // nodes g .. g + 3 (up to the last)
+    float2 edge;        // C_0 of the lower half, Q_last of the upper
+    float2 w[NODES];    // nodes g .. g + NODES - 1 (up to the last)
     int g;
 };
 
@@ -210,7 +211,8 @@ __device__ __forceinline__ bool key_past(bool lower, df2 key, float2 v)
     return lower ? d > 0.0f : d < 0.0f;
 }
 
-__device__ __forceinline__ FracPair row_invert_f(const RowWindow &r, const float2 *__restrict__ V,
+template <int NODES>
+__device__ __forceinline__ FracPair row_invert_f(const RowWindow<NODES> &r, const float2 *__restrict__ V,
                                                  const float *__restrict__ En, bool lower, df2 key,
                                                  float ds, bool power_tail)
 {
@@ -219,11 +221,11 @@ __device__ __forceinline__ FracPair row_invert_f(const RowWindow &r, const float
     if (lo < kNNode - 2 && key_past(lower, key, c_hi)) {
         ++lo;
         c_lo = c_hi;
-        c_hi = r.w[2];
+        c_hi = NODES > 2 ? r.w[NODES > 2 ? 2 : 0] : ldg2(V + lo + 1);
         if (lo < kNNode - 2 && key_past(lower, key, c_hi)) {
             ++lo;
             c_lo = c_hi;
-            c_hi = r.w[3];
+            c_hi = NODES > 3 ? r.w[NODES > 3 ? 3 : 0] : ldg2(V + lo + 1);
 #pragma unroll 1
             while (lo < kNNode - 2 && key_past(lower, key, c_hi)) {
                 ++lo;
@@ -256,6 +258,7 @@ __device__ __forceinline__ FracPair row_invert_f(const RowWindow &r, const float
 
 // Inverse CDF of Eq. 7 (emission rows) or of the pair spectrum, linear
 // between the two chi rows around chi (same rule as the FP64 path).
+template <int NODES>
 __device__ __forceinline__ FracPair sample_cdf_f(const float2 *__restrict__ rows,
                                                  const float2 *__restrict__ qrows,
                                                  const unsigned char *__restrict__ guide,
@@ -281,7 +284,7 @@ __device__ __forceinline__ FracPair sample_cdf_f(const float2 *__restrict__ rows
                               guide_bucket(key.hi);
     // a single row is read as both of a pair
     const int dn = nrow == 2 ? kNNode : 0, dg = nrow == 2 ? kGuideBuckets : 0;
-    RowWindow r[2];
+    RowWindow<NODES> r[2];
     r[0].g = (int)__ldg(gd);
     r[1].g = (int)__ldg(gd + dg);
     r[0].edge = ldg2(V + (lower ? 0 : kNNode - 1));
@@ -289,7 +292,7 @@ __device__ __forceinline__ FracPair sample_cdf_f(const float2 *__restrict__ rows
 #pragma unroll
     for (int k = 0; k < 2; ++k)
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < NODES; ++i)
             r[k].w[i] = ldg2(V + k * dn + min(r[k].g + i, kNNode - 1));
     const FracPair a = row_invert_f(r[0], V, En, lower, key, ds, emission);
     if (nrow == 2) {

@@ -420,13 +420,25 @@ __device__ __forceinline__ void mid_get(const R (*w)[kQueue], int t, R b0, Lepto
     }
 }
 
-// Shared-memory layout of k_step (dynamic part).
+// Short tiles of the mixed path on a 2D grid run their emitters in place: a
+// lepton there carries six field components to them, and a push whose gather
+// keeps 24 loads in flight has no registers for it (2D foil: 36 us a step in
+// place, 38.5 packed).  The kernels of 2D grids have no long tiles either
+// (has_long_tiles): the call alone costs them registers (39.5 us).
+template <int FK, typename R>
+constexpr bool kEmitInPlace = sizeof(R) == 4 && FK == QP_FIELD_YEE2D;
+
+// Shared-memory layout of k_step (dynamic part).  Where emitters run in place
+// nothing is queued: the 12 KB a block are left to the L1 cache, which serves
+// the gather.
 template <int FK, typename R>
 struct Smem {
+    static constexpr bool kQueued = !kEmitInPlace<FK, R>;
     R H[kNRatePad];                          // rate tables (TMA-staged)
     R G[kNRatePad];
     R T[kNRatePad];
-    R mid[kWarps][mid_words<FK>()][kQueue];  // each warp's emitters
+    // each warp's emitters
+    R mid[kQueued ? kWarps : 1][kQueued ? mid_words<FK>() : 1][kQueue];
 };
 
 __device__ __forceinline__ void wait_tables(unsigned long long *bar, const StepArgs &a)
@@ -688,6 +700,11 @@ __device__ __forceinline__ void lepton_finish(const Problem &P, const LeptonStat
     }
 }
 
+// Nodes of a CDF row that a sample loads at once (mixed path): on a 2D grid the
+// gather's values leave registers for fewer.
+template <int FK>
+constexpr int kWindowNodes = FK == QP_FIELD_YEE2D ? 3 : 4;
+
 template <int PREC, int FK, typename R, class Sink>
 __device__ __forceinline__ void lepton_events(const StepArgs &a, const Problem &P,
                                               const StepTime &tm, const R *H, int sp, const SpeciesDev &S, int64_t i,
@@ -765,7 +782,7 @@ __device__ __forceinline__ void lepton_events(const StepArgs &a, const Problem &
             // ---- emission: Eq. 7 sampling, Eq. 8 recoil
             const uint4 rr = draw(P.seed, sp, kRngEmit, particle_id(S, i), tm.step, k);
             const float xi = u53f(rr.z, rr.w);
-            const FracPair uf = sample_cdf_f(
+            const FracPair uf = sample_cdf_f<kWindowNodes<FK>>(
                 a.tab.Cg2, a.tab.Qg2, a.tab.Gg, a.tab.Eg, chi, u53_pair(rr.x, rr.y),
                 u53_pair_complement(rr.x, rr.y), (float)(kSgSpan / (kNNode - 1)), true, clamped);
             const float pmag = sqrtf(ux * ux + uy * uy + uz * uz);
@@ -927,14 +944,6 @@ constexpr int kPart = 32 * kSubTiles, kLongTile = kPart * kWarps;
 constexpr int kShortShift = 7, kLongShift = 10;
 static_assert((1 << kShortShift) == kTile && (1 << kLongShift) == kLongTile, "tile sizes");
 constexpr int kTickets = 2 * kRing;
-
-// Short tiles of the mixed path on a 2D grid run their emitters in place: a
-// lepton there carries six field components to them, and a push whose gather
-// keeps 24 loads in flight has no registers for it (2D foil: 36 us a step in
-// place, 38.5 packed).  The kernels of 2D grids have no long tiles either
-// (has_long_tiles): the call alone costs them registers (39.5 us).
-template <int PREC, int FK>
-constexpr bool kEmitInPlace = PREC != kFP64 && FK == QP_FIELD_YEE2D;
 
 // The emission loop of the lepton in slot i, its record number e of the stash;
 // wgt: its weight.
@@ -1222,7 +1231,7 @@ __device__ __forceinline__ bool photon_step(const StepArgs &a, const Problem &P,
 // optical depths are sampled here (Eq. 7), on packed lanes, from the chi in
 // the stash and the photon's slot, which nothing has touched since it
 // decayed.
-template <int PREC, class Record>
+template <int PREC, int NODES, class Record>
 __device__ __forceinline__ void write_pairs(const StepArgs &a, const Problem &P,
                                             const StepTime &tm, int n,
                                             Record record, long long excl, long long be,
@@ -1250,7 +1259,7 @@ __device__ __forceinline__ void write_pairs(const StepArgs &a, const Problem &P,
                 tm = -log(u53(r1.z, r1.w));
                 tp = -log(u53(r2.x, r2.y));
             } else {
-                const FracPair vf = sample_cdf_f(
+                const FracPair vf = sample_cdf_f<NODES>(
                     a.tab.Cp2, a.tab.Qp2, a.tab.Gp, a.tab.Ep, hi_d(chi), u53_pair(r1.x, r1.y),
                     u53_pair_complement(r1.x, r1.y), (float)(kSpSpan / (kNNode - 1)), false,
                     clamped);
@@ -1353,17 +1362,25 @@ __device__ __forceinline__ ProbCounts problem_counts(const Problem &P)
     return c;
 }
 
-// The step's index and time, and the FP32 / double-float time constants of the
-// mixed path.
+// The step's index, and its time as the field reads it: FP64, or the mixed path's
+// double-float constants (a 2D grid and a constant field need none).
+template <int PREC, int FK>
 __device__ __forceinline__ void set_time(StepTime &tm, const Problem &P, long long step)
 {
     tm.step = (uint64_t)step;
-    tm.t = (double)step * P.dt;
-    const double tr = tm.t - P.f.t_focus;
-    tm.t_hi = __double2float_rn(tm.t);
-    tm.t_lo = __double2float_rn(tm.t - (double)tm.t_hi);
-    tm.tr_hi = __double2float_rn(tr);
-    tm.tr_lo = __double2float_rn(tr - (double)tm.tr_hi);
+    if constexpr (FK == QP_FIELD_PLANE || FK == QP_FIELD_GAUSSIAN) {
+        const double t = __dmul_rn((double)step, P.dt);  // (rounded: no sum may take it in)
+        if constexpr (PREC == kFP64) {
+            tm.t = t;
+        } else if constexpr (FK == QP_FIELD_PLANE) {
+            tm.t_hi = __double2float_rn(t);
+            tm.t_lo = __double2float_rn(t - (double)tm.t_hi);
+        } else {
+            const double tr = t - P.f.t_focus;
+            tm.tr_hi = __double2float_rn(tr);
+            tm.tr_lo = __double2float_rn(tr - (double)tm.tr_hi);
+        }
+    }
 }
 
 // Block-wide inclusive scan of v[0..n) in place (n <= 2 kTile).
@@ -1466,7 +1483,7 @@ __device__ __forceinline__ bool short_leptons(const StepArgs &a, const Problem &
         event = lepton_push<PREC, FK, R>(a, P, tm, sm.H, sm.G, sp, s, mid, o, sink);
         if (!event)
             lepton_finish<PREC, R>(P, s, mid, sink);
-        else if constexpr (kEmitInPlace<PREC, FK>)
+        else if constexpr (kEmitInPlace<FK, R>)
             run_emitter<PREC, FK, R>(a, P, tm, sm.H, sp, i, s, mid, st, kTile, tid, o, wgt);
         else
             mid_put<FK, R>(sm.mid[tid >> 5], (int)half + (tid & 31), mid);
@@ -1481,7 +1498,7 @@ __device__ __forceinline__ bool short_leptons(const StepArgs &a, const Problem &
     }
     warp_count(&bs.c[sp][cCont], o.cont);
     warp_count(&bs.c[sp][cClamp], o.clamped);
-    if (kEmitInPlace<PREC, FK> && __any_sync(0xFFFFFFFFu, event)) {
+    if (kEmitInPlace<FK, R> && __any_sync(0xFFFFFFFFu, event)) {
         const int photons = count_emitters(bs, sp, o, wgt);
         if ((tid & 31) == 0) atomicAdd(&rec.made, photons);
     }
@@ -1591,7 +1608,7 @@ __device__ __forceinline__ void set_pending(const StepArgs &a, const Problem &P,
 // A tile's prefix is resolved (its predecessors are, by now, almost always
 // published) and its photons or pairs are written, by one warp.  HERE: its
 // emitters ran in place.
-template <int PREC, bool HERE>
+template <int PREC, int FK, bool HERE>
 __device__ __forceinline__ void flush_short(const StepArgs &a, const Problem &P,
                                             const ProbCounts &pc, const ShortRec &rec,
                                             const StepTime &tm, unsigned epoch, BlockStats &bs, const double *st)
@@ -1607,7 +1624,7 @@ __device__ __forceinline__ void flush_short(const StepArgs &a, const Problem &P,
             [&](int e) { return HERE ? (int)rec.list[listed_entry(rec, e)] : e; },
             pc.n[2] + excl, bs);
     else
-        write_pairs<PREC>(
+        write_pairs<PREC, kWindowNodes<FK>>(
             a, P, tm, total,
             [&](int e, int64_t &i) {
                 const int t = rec.list[listed_entry(rec, e)];
@@ -1759,7 +1776,7 @@ __device__ __forceinline__ int photon_part(const StepArgs &a, const Problem &P,
 // by the first warp of the block to come here (its predecessors are, by now,
 // almost always published), then every warp writes its own photons or pairs
 // behind the parts before it.
-template <int PREC>
+template <int PREC, int FK>
 __device__ __forceinline__ void flush_part(const StepArgs &a, const Problem &P,
                                            const StepTime &tm,
                                            const ProbCounts &pc, const PartRec &part,
@@ -1800,7 +1817,7 @@ __device__ __forceinline__ void flush_part(const StepArgs &a, const Problem &P,
                 write_photons<PREC>(P, tm, part.sp, part.n, st, kPart, [](int e) { return e; },
                                     pc.n[2] + excl, bs);
             else
-                write_pairs<PREC>(
+                write_pairs<PREC, kWindowNodes<FK>>(
                     a, P, tm, part.n,
                     [&](int e, int64_t &i) {
                         i = __double_as_longlong(st[kStashSlot * kPart + e]);
@@ -1840,7 +1857,8 @@ struct StepShared {
             PartRec part[kWarps][kRing];
         } lng;
     } ring;
-    unsigned slots[kWarps][kQueue];   // long: slots of the queued emitters
+    // long: slots of the queued emitters
+    unsigned slots[has_long_tiles(FK) ? kWarps : 1][has_long_tiles(FK) ? kQueue : 1];
     alignas(16) Problem prob;         // batch, or long: the problem of the current tile
 };
 
@@ -1871,7 +1889,7 @@ __device__ __forceinline__ void leave_problem(const StepArgs &a, const Problem &
 }
 
 // Problem b takes its place in shared memory, cut into long or short tiles.
-template <int FK, typename R>
+template <int PREC, int FK, typename R>
 __device__ __forceinline__ void enter_problem(StepShared<FK, R> &sh, const Problem &src, bool lng)
 {
     const int *from = reinterpret_cast<const int *>(&src);
@@ -1884,7 +1902,7 @@ __device__ __forceinline__ void enter_problem(StepShared<FK, R> &sh, const Probl
         sh.pc = problem_counts(sh.prob);
         sh.pc.set_tiles(lng);
         if (sh.prob.device_step)
-            set_time(sh.tm, sh.prob, *((volatile long long *)sh.prob.step_ctr));
+            set_time<PREC, FK>(sh.tm, sh.prob, *((volatile long long *)sh.prob.step_ctr));
     }
     __syncthreads();
 }
@@ -1974,7 +1992,7 @@ __device__ __noinline__ void long_tile_loop(const StepArgs &a, const Problem *ta
         const unsigned upto = leave ? n : n + 1u > (unsigned)kLag ? n + 1u - (unsigned)kLag : 0u;
 #pragma unroll 1
         for (; lo < upto; ++lo)
-            flush_part<PREC>(a, P, tm, sh.pc, sh.ring.lng.part[warp][lo % kRing],
+            flush_part<PREC, FK>(a, P, tm, sh.pc, sh.ring.lng.part[warp][lo % kRing],
                              sh.ring.lng.rec[lo % kRing], lo, warp, epoch, bs, part_stash(lo));
         if (!leave) {
             ++n;
@@ -1982,7 +2000,7 @@ __device__ __noinline__ void long_tile_loop(const StepArgs &a, const Problem *ta
         }
         leave_problem(a, P, cur, bs);
         if (!more) break;
-        enter_problem<FK, R>(sh, table[b], true);
+        enter_problem<PREC, FK, R>(sh, table[b], true);
         cur = b;
     }
     // the copies of the tables land before the block leaves
@@ -2073,7 +2091,7 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
         sh.tdone = 1u;
         sh.tclaim = sh.claim = 0u;
     }
-    if (!BATCH && tid == 97) set_time(sh.tm, a.single, (long long)a.single.step + step);
+    if (!BATCH && tid == 97) set_time<PREC, FK>(sh.tm, a.single, (long long)a.single.step + step);
     if (tid >= 32 && tid < 64)
         for (int k = tid - 32; k < (int)(sizeof(sh.ring) / sizeof(int)); k += 32)
             reinterpret_cast<int *>(&sh.ring)[k] = 0;
@@ -2119,7 +2137,7 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
     const long long n_tickets = sh.off[np - 1];
     if (!lng) {
         int cur = BATCH ? -1 : 0;
-        constexpr bool kHere = kEmitInPlace<PREC, FK>;
+        constexpr bool kHere = kEmitInPlace<FK, R>;
         // tiles of this block, counted from its first (uniform over the
         // block): q started, q_ev with their events resolved (q or q - 1),
         // q_lo written
@@ -2136,7 +2154,7 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
                     leave_problem(a, BATCH ? sh.prob : a.single, cur, bs);
                 if (!more) break;
                 if constexpr (BATCH) {
-                    enter_problem<FK, R>(sh, table[b], false);
+                    enter_problem<PREC, FK, R>(sh, table[b], false);
                     cur = b;
                 }
             }
@@ -2193,12 +2211,14 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
 
             // ---- the previous tile's emitters
             bool finished = false;  // this warp finished them
-            if (!kHere && q_ev != q) {
-                ShortRec &rec = sh.ring.shrt[q_ev % kRing];
-                if (rec.chain == 0)
-                    finished = resolve_emitters<PREC, FK, R>(
-                        a, P, tm, sm, rec, (q_ev & 1u) * 32u, drain, epoch, bs,
-                        stash + (size_t)(q_ev % kRing) * kStashFieldsHost * kTile);
+            if constexpr (!kHere) {
+                if (q_ev != q) {
+                    ShortRec &rec = sh.ring.shrt[q_ev % kRing];
+                    if (rec.chain == 0)
+                        finished = resolve_emitters<PREC, FK, R>(
+                            a, P, tm, sm, rec, (q_ev & 1u) * 32u, drain, epoch, bs,
+                            stash + (size_t)(q_ev % kRing) * kStashFieldsHost * kTile);
+                }
             }
 
             // ---- during a problem the first warp to come here writes the
@@ -2222,7 +2242,7 @@ __global__ void __launch_bounds__(kTile, step_min_blocks<PREC, FK>())
 #pragma unroll 1
             for (;; now = after, after = -1) {
                 if (now >= 0)
-                    flush_short<PREC, kHere>(a, P, sh.pc, sh.ring.shrt[now], tm, epoch, bs,
+                    flush_short<PREC, FK, kHere>(a, P, sh.pc, sh.ring.shrt[now], tm, epoch, bs,
                                       stash + (size_t)now * kStashFieldsHost * kTile);
                 if (after < 0) break;
             }
@@ -2398,7 +2418,7 @@ __global__ void __launch_bounds__(32, 32) k_fused(const __grid_constant__ FusedA
             const int *src = reinterpret_cast<const int *>(&a.single);
             int *dst = reinterpret_cast<int *>(&sP);
             for (int k = lane; k < (int)(sizeof(Problem) / sizeof(int)); k += 32) dst[k] = src[k];
-            if (lane == 0) set_time(tm, a.single, (long long)a.single.step);
+            if (lane == 0) set_time<PREC, FK>(tm, a.single, (long long)a.single.step);
         }
         __syncwarp();
         const int sp = tile < f.tiles_e ? 0 : 1;
@@ -2424,7 +2444,7 @@ __global__ void __launch_bounds__(32, 32) k_fused(const __grid_constant__ FusedA
         for (int k = 0; k < f.K; ++k) {
             if (k > 0) {
                 __syncwarp();
-                if (lane == 0) set_time(tm, sP, (long long)(s0 + k));
+                if (lane == 0) set_time<PREC, FK>(tm, sP, (long long)(s0 + k));
                 __syncwarp();
             }
             LeptonOut o{};
