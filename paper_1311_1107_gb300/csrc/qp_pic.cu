@@ -214,12 +214,20 @@ __global__ void __launch_bounds__(kPicBlock) k_deposit(SpeciesDev A, SpeciesDev 
     }
     const int64_t stride = (int64_t)blocks * blockDim.x;
     float *J[3] = {jx, jy, jz};
-    // Neighbours in a sorted species share a cell: the lanes of a warp take
-    // every eighth of the block's slots, so that an atomic add meets fewer equal
-    // addresses, and the block's warps share the lines that they read (137000
-    // leptons at 8 a cell: 10.1 -> 8.9 us; 16-byte vector adds: 9.2).
-    constexpr int kWarps = kPicBlock / 32;
-    const int slot = (threadIdx.x & 31) * kWarps + (threadIdx.x >> 5);
+    // Neighbours in a sorted species share a cell: the lanes of a warp take every
+    // kSpread-th of the slots of kSpread warps, so that an atomic add meets fewer
+    // equal addresses and those warps share the lines that they read.  More of it
+    // costs a species that has moved since its sort, whose warps then add to
+    // more lines.  Us a call, kSpread 1 / 2 / 4 / 8:
+    //                                  sorted              moved by 1.5 cells rms
+    //   131072 leptons, 8 a cell   7.2/ 6.0/ 5.9/ 6.1      8.7/ 8.6/ 9.1/10.0
+    //   131072 leptons, 4 a cell   6.7/ 6.4/ 6.4/ 7.3      8.7/ 9.2/10.3/12.1
+    //   1.05e6 leptons, 8 a cell  45.7/33.6/32.9/36.1     59.3/58.9/61.4/71.9
+    // (16-byte vector adds instead: 9.2 where the spread over 8 took 8.9.)
+    constexpr int kSpread = 2;
+    static_assert(kPicBlock / 32 % kSpread == 0, "whole groups of warps");
+    const int warp = threadIdx.x >> 5;
+    const int slot = warp / kSpread * (32 * kSpread) + (threadIdx.x & 31) * kSpread + warp % kSpread;
     for (int64_t p = (int64_t)block * blockDim.x + slot; p < n; p += stride) {
         const double xd = S.x[p], yd = S.y[p], uxd = S.ux[p], uyd = S.uy[p], uzd = S.uz[p],
                      wd = S.w[p];
