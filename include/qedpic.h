@@ -224,7 +224,9 @@ typedef struct {
  * the first of a path, or of capacities that fill every warp several times
  * over, its append scratch (74 MB, then up to 444 MB): an allocation each,
  * synchronous; otherwise no allocation, no host synchronisation,
- * no host reads: the call can then be captured in a CUDA graph.  Up to eight
+ * no host reads: the call can then be captured in a CUDA graph.  Where the
+ * larger append scratch cannot be had (during a capture, or short of memory)
+ * the steps do without it, slower and with the same results.  Up to eight
  * steps (one while launches are timed, see qp_profile_enable) are one launch
  * of the step kernel over every resident block of the GPU; on the mixed path,
  * and for more than one step, it is a cooperative launch, which starts only
@@ -233,7 +235,8 @@ typedef struct {
  * Returns QP_ERR_INVALID_ARG (nothing enqueued) for bad parameters, a
  * missing photon species while species emit, or a YEE2D grid with a NULL
  * component; QP_ERR_CUDA if a launch fails.  Overflow, table clamping and
- * wait time-outs are reported by the next qp_diagnostics.
+ * wait time-outs are reported by the next qp_diagnostics; after a time-out
+ * the steps left in its launch are not published.
  */
 int qp_step(qp_ctx *ctx, const qp_step_params *s, void *stream);
 

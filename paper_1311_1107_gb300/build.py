@@ -25,7 +25,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # Per-unit flags.  The mixed-precision step divides in FP32 with the
 # hardware reciprocal (2 ulp): its tolerance is set by FP32 physics, and the
 # IEEE division's range checks and slow path cost more than the division.
-# The FP64 step keeps IEEE arithmetic throughout.
+# The FP64 step keeps IEEE division and square root where it calls them; most of
+# its quotients and roots are Newton iterations within a unit of the last place.
 # The coalescence forms its groups and sums with the oracle's FP64
 # operations in the oracle's order: no FMA contraction there.
 UNIT_FLAGS = {"qp_step_mixed.cu": ["-prec-div=false"], "qp_coalesce.cu": ["-fmad=false"]}

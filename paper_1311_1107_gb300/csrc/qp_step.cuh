@@ -212,7 +212,7 @@ __device__ __noinline__ long long spread_ticket(StepCtl *ctl, unsigned limit, in
 // Decoupled look-back over a chain of tiles.  A tile first publishes its
 // aggregate (the number of particles it appends); the exclusive prefix is
 // then computed by one full warp with a 32-tile window: lane l inspects tile
-// base - l; a word counts only if it carries this launch's epoch.  The
+// base - l; a word counts only if it carries this step's epoch.  The
 // window is consumed up to the nearest tile that published its inclusive
 // prefix, summing the aggregates in between.  Waits are bounded by
 // spin_limit; on time-out the status is raised and the prefix is what was
@@ -1322,8 +1322,8 @@ __device__ __forceinline__ int step_photons(const StepArgs &a, const Problem &P,
 
 // -------------------------------------------------------------------- the step
 
-// Live slots of one problem for this launch, and its long or short tiles.  Live
-// counts and step counters change only at the end of a launch (last block),
+// Live slots of one problem in this step, and its long or short tiles.  Live
+// counts and step counters change only at the end of a step (last block),
 // so every block sees the same values.  Counts outside [0, capacity] are
 // clamped (and reported).
 struct ProbCounts {
@@ -1583,7 +1583,7 @@ __device__ __forceinline__ long long pair_room(const Problem &P, const ProbCount
 }
 
 // The live counts after the last tile of a chain, whose particles are number
-// excl .. excl + total - 1 (applied at the end of the launch).
+// excl .. excl + total - 1 (applied at the end of the step).
 __device__ __forceinline__ void set_pending(const StepArgs &a, const Problem &P,
                                             const ProbCounts &pc, int chain, long long excl,
                                             int total)
@@ -1842,9 +1842,9 @@ struct StepShared {
     long long ticket[kTickets];       // ticket of tile n at n % kTickets
     unsigned tdone, tclaim;           // long: tiles with a ticket; being fetched
     unsigned claim;                   // short: warps that asked to flush
-    int last, go;                     // the launch's last block; its next step has begun
+    int last, go;                     // the step's last block; the next step has begun
     long long tmp[kWarps];
-    unsigned long long subs;          // 32-slot sub-tiles of the launch
+    unsigned long long subs;          // 32-slot sub-tiles of the step
     BlockStats bs;
     StepTime tm;                      // of the current problem's step
     ProbCounts pc;                    // of the current problem
@@ -2008,9 +2008,10 @@ __device__ __noinline__ void long_tile_loop(const StepArgs &a, const Problem *ta
     if (!ph_loaded) wait_tables(&sh.bar[1], a);
 }
 
-// One launch = one step of every active problem.  Persistent blocks take
-// tiles by ticket (a block's first tile is fixed in a cooperative launch, every
-// other ticket comes from an atomic counter, fetched while the tile before it
+// One launch = one step of every active problem of a batch, or one to
+// kStepsPerLaunch steps of a single problem.  Persistent blocks take
+// tiles by ticket (a block's first tile of a step is fixed in a cooperative
+// launch, every other ticket comes from an atomic counter, fetched while the tile before it
 // runs); tickets enumerate, problem after problem, its electron tiles,
 // positron tiles and photon tiles, so within each problem's chains start
 // order is tile order and the decoupled look-back only ever waits on tiles
